@@ -825,7 +825,7 @@ rsrr_status rsrr_sample_batch(rsrr_t *const *handles, int32_t count, void *strea
         rsrr::thread_error() = std::string("rsrr_sample_batch: grouped band LU: ") + cudaGetErrorString(e);
         return RSRR_ECUDA;
     }
-    hs_[0]->launches += (t64.empty() ? 0 : 1) + (t128.empty() ? 0 : 1);
+    hs_[0]->launches += (t64.empty() ? 0 : 2) + (t128.empty() ? 0 : 2);
     for (Handle *h : hs_) {
         rsrr_status st = h->sample_band(0, h->N, s, 2);
         if (st != RSRR_OK) return st;
@@ -1426,7 +1426,7 @@ rsrr_status Handle::sample_band(int p0, int np, cudaStream_t s, int phase) {
         CK(launch_widen_r32(X, D, per_pt * np, s), "widen");
         CK(cudaMemsetAsync(done, 0, sizeof(int32_t) * np, s), "memset");
         if ((ms = mark(3, s)) != RSRR_OK) return ms;
-        launches += 5;  // assemble, LU, probe, solve, widen
+        launches += 6;  // assemble, LU, U11 inverses, probe, solve, widen
         for (int it = 0; it < opts.max_refine; ++it) {
             CK(launch_residual(R, X, dq, rmax, xmax, done, s), "residual");
             CK(launch_eta(eta, done, rmax, xmax, d_umax, tnorm, np, L, opts.eta_tol, d_sweep_flags + it, done, s),
@@ -1448,7 +1448,7 @@ rsrr_status Handle::sample_band(int p0, int np, cudaStream_t s, int phase) {
         CK(real_solve(false, D, nullptr, p0, np, s), "band solve");
         CK(launch_widen_r64(X, D, per_pt * np, s), "widen");
         if ((ms = mark(3, s)) != RSRR_OK) return ms;
-        launches += 5;  // assemble, LU, probe, solve, widen
+        launches += 6;  // assemble, LU, U11 inverses, probe, solve, widen
     } else if (opts.precision == RSRR_PREC_MIXED) {
         float2 *ab = d_ab32 + fo(p0) * ab_pt, *D = d_D + fo(p0) * per_pt;
         double2 *R = d_R + fo(p0) * per_pt;
@@ -1464,7 +1464,7 @@ rsrr_status Handle::sample_band(int p0, int np, cudaStream_t s, int phase) {
         CK(launch_widen(X, D, per_pt * np, s), "widen");
         CK(cudaMemsetAsync(done, 0, sizeof(int32_t) * np, s), "memset");
         if ((ms = mark(3, s)) != RSRR_OK) return ms;
-        launches += 5;  // assemble, LU, probe, solve, widen
+        launches += 6;  // assemble, LU, U11 inverses, probe, solve, widen
         if (opts.refine == RSRR_REFINE_GMRES) {
             if ((ms = refine_gmres(p0, np, dq, s)) != RSRR_OK) return ms;
         } else
@@ -1489,7 +1489,7 @@ rsrr_status Handle::sample_band(int p0, int np, cudaStream_t s, int phase) {
         CK(launch_broadcast_probe_c128(X, d_U, per_pt, np, s), "probe");
         CK(band_solve(false, X, nullptr, p0, np, s), "band solve");
         if ((ms = mark(3, s)) != RSRR_OK) return ms;
-        launches += 4;  // assemble, LU, probe, solve
+        launches += 5;  // assemble, LU, U11 inverses, probe, solve
     }
     if ((ms = mark(4, s)) != RSRR_OK) return ms;
     // final backward errors of every column of the range (statistics and
