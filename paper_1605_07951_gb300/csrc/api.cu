@@ -1874,31 +1874,35 @@ bool Handle::dense_residual_sliced() const {
 }
 
 // R = U - T X in FP64 (stored complex128 T) and the column maxima of |R|, |X|,
-// for points p0 .. p0+np-1, or (skip_done) only for those whose done flag is 0
-// (the flags are read on the host first).
+// for points p0 .. p0+np-1, or (skip_done) only for those whose done flag is 0.
+// Products large enough for the sliced tensor-core GEMM run point by point (the
+// flags are read on the host first); the others in one launch over the points.
 rsrr_status Handle::dense_residual(bool skip_done, int p0, int np, cudaStream_t s) {
     Handle *h = this;
-    std::vector<int32_t> done(np, 0);
-    if (skip_done) {
-        CK(cudaMemcpyAsync(done.data(), d_done + p0, sizeof(int32_t) * np, cudaMemcpyDeviceToHost, s), "done");
-        CK(cudaStreamSynchronize(s), "done sync");
-    }
     const size_t per = (size_t)n * L, nn2 = (size_t)n * n;
-    for (int q = 0; q < np; ++q) {
-        if (done[q]) continue;
-        const size_t pt = (size_t)p0 + q;
-        CK(cudaMemcpyAsync(d_R + pt * per, d_U, sizeof(double2) * per, cudaMemcpyDeviceToDevice, s), "R = U");
-        if (dense_residual_sliced())
+    const int32_t *flags = skip_done ? d_done + p0 : nullptr;
+    if (!dense_residual_sliced()) {
+        CK(launch_dense_residual(d_R + p0 * per, d_T64 + p0 * nn2, d_X + p0 * per, d_U, (int)n, L, np, flags, s),
+           "R = U - T X");
+        launches += 1;
+    } else {
+        std::vector<int32_t> done(np, 0);
+        if (skip_done) {
+            CK(cudaMemcpyAsync(done.data(), flags, sizeof(int32_t) * np, cudaMemcpyDeviceToHost, s), "done");
+            CK(cudaStreamSynchronize(s), "done sync");
+        }
+        for (int q = 0; q < np; ++q) {
+            if (done[q]) continue;
+            const size_t pt = (size_t)p0 + q;
+            CK(cudaMemcpyAsync(d_R + pt * per, d_U, sizeof(double2) * per, cudaMemcpyDeviceToDevice, s), "R = U");
             CK(ozaki_zgemm((int)n, L, (int)n, false, d_T64 + pt * nn2, n, d_X + pt * per, n, d_R + pt * per, n,
                            -1.0, 1.0, false, d_dws, dws_bytes, s, &launches, nullptr, nullptr,
                            opts.gemm == RSRR_GEMM_OZAKI_MMA, d_tmo), "R -= T X");
-        else
-            CK(fp64_gemm((int)n, L, (int)n, false, d_T64 + pt * nn2, n, d_X + pt * per, n, d_R + pt * per, n,
-                         -1.0, 1.0, s), "R -= T X");
-        CK(launch_dense_colmax(d_R + pt * per, d_X + pt * per, (int)n, L, d_rmax + pt * L, d_xmax + pt * L, s),
-           "colmax");
-        launches += 2;
+        }
     }
+    CK(launch_dense_colmax(d_R + p0 * per, d_X + p0 * per, (int)n, L, np, d_rmax + (size_t)p0 * L,
+                           d_xmax + (size_t)p0 * L, flags, s), "colmax");
+    launches += 1;
     return RSRR_OK;
 }
 

@@ -147,8 +147,10 @@ cudaError_t launch_dense_solve_c64(const float2 *A, const int32_t *piv, const fl
 cudaError_t launch_dense_solve_c128(const double2 *A, const int32_t *piv, const double2 *dinv,
                                     double2 *B, int n, int N, int L, const int32_t *skip,
                                     cudaStream_t s);
-cudaError_t launch_dense_colmax(const double2 *R, const double2 *X, int n, int L, double *rmax,
-                                double *xmax, cudaStream_t s);
+cudaError_t launch_dense_residual(double2 *R, const double2 *T, const double2 *X, const double2 *U, int n, int L,
+                                  int N, const int32_t *done, cudaStream_t s);
+cudaError_t launch_dense_colmax(const double2 *R, const double2 *X, int n, int L, int N, double *rmax,
+                                double *xmax, const int32_t *done, cudaStream_t s);
 cudaError_t launch_taylor_step(double2 *A, const double *pts, double2 c, double diag, int n, int p,
                                cudaStream_t s);
 cudaError_t launch_dense_eig_residual(const double2 *V, const double2 *lam, const double *pts,
