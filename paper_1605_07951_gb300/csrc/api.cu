@@ -985,7 +985,7 @@ rsrr_status Handle::allocate_and_upload(const std::vector<double2> &coef) {
         use_solve2 = solve2;
         cluster_lu = !(opts.flags & RSRR_FLAG_ONE_CTA_LU);
         if (solve2) {
-            CK(alloc(&d_bperm, (size_t)fcap * ((n + geom.nb - 1) / geom.nb) * 2 * geom.nb),
+            CK(alloc(&d_bperm, (size_t)fcap * ((n + geom.nb - 1) / geom.nb) * bp_ints(geom.nb)),
                "alloc block permutations");
             CK(alloc(&d_gate, 1), "alloc");
         }
@@ -1056,7 +1056,7 @@ cudaError_t Handle::band_solve(bool mixed, void *B, const int32_t *skip, int p0,
     const int nn = (int)n;
     const size_t ab_pt = (size_t)geom.ldab * n;
     const size_t nblk = ((size_t)n + geom.nb - 1) / geom.nb;
-    const size_t bp_pt = nblk * 2 * geom.nb, dv_pt = nblk * 2 * geom.nb * geom.nb;
+    const size_t bp_pt = nblk * bp_ints(geom.nb), dv_pt = nblk * 2 * geom.nb * geom.nb;
     if (mixed)
         return use_solve2 ? launch_band_solve2_c64(d_ab32 + fo(p0) * ab_pt, d_bperm + fo(p0) * bp_pt, d_dinv32 + fo(p0) * dv_pt,
                                                static_cast<float2 *>(B), geom, np, nn, L, skip, s)
@@ -1074,7 +1074,7 @@ cudaError_t Handle::real_solve(bool mixed, void *B, const int32_t *skip, int p0,
     const int nn = (int)n;
     const size_t ab_pt = (size_t)geom.ldab * n;
     const size_t nblk = ((size_t)n + geom.nb - 1) / geom.nb;
-    const size_t bp_pt = nblk * 2 * geom.nb, dv_pt = nblk * 2 * geom.nb * geom.nb;
+    const size_t bp_pt = nblk * bp_ints(geom.nb), dv_pt = nblk * 2 * geom.nb * geom.nb;
     if (mixed)
         return use_solve2 ? launch_band_solve2_r32(d_abr32 + fo(p0) * ab_pt, d_bperm + fo(p0) * bp_pt, d_dinvr32 + fo(p0) * dv_pt,
                                                    static_cast<float *>(B), geom, np, nn, L, skip, s)
@@ -1087,14 +1087,16 @@ cudaError_t Handle::real_solve(bool mixed, void *B, const int32_t *skip, int p0,
 }
 
 cudaError_t Handle::sweep_solve(float2 *B, const int32_t *skip, int p0, int np, cudaStream_t s) {
-    if (!use_solve2 || !d_gate || (opts.flags & RSRR_FLAG_WIDE_SOLVE_ONLY)) return band_solve(true, B, skip, p0, np, s);
+    if (!use_solve2 || !d_gate) return band_solve(true, B, skip, p0, np, s);
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t ab_pt = (size_t)geom.ldab * n;
     const size_t nblk = ((size_t)n + geom.nb - 1) / geom.nb;
-    const size_t bp_pt = nblk * 2 * geom.nb, dv_pt = nblk * 2 * geom.nb * geom.nb;
+    const size_t bp_pt = nblk * bp_ints(geom.nb), dv_pt = nblk * 2 * geom.nb * geom.nb;
     const float2 *ab = d_ab32 + fo(p0) * ab_pt, *dv = d_dinv32 + fo(p0) * dv_pt;
     const int32_t *bp = d_bperm + fo(p0) * bp_pt;
+    if (opts.flags & RSRR_FLAG_WIDE_SOLVE_ONLY)
+        return launch_band_solve2_c64(ab, bp, dv, B, geom, np, (int)n, L, skip, s, 16);
     // the device picks the shape (16, 8, 4 or 2 right-hand sides per CTA)
     // from the points still active; the other three launches return at once
     cudaError_t e = launch_solve_gate(skip, np, L, sms, d_gate, s);
@@ -1301,7 +1303,7 @@ rsrr_status Handle::autotune(cudaStream_t s) {
         launches += 2;
     }
     if (solve2) {
-        CK(launch_block_perm(d_bperm, d_piv, nn, geom.kl, geom.nb, N, s), "tune block permutations");
+        CK(launch_block_perm(d_bperm, d_piv, nn, geom.kl, geom.ku, geom.nb, N, s), "tune block permutations");
         launches += 1;
     }
     const bool save = use_solve2;
@@ -1383,7 +1385,7 @@ rsrr_status Handle::sample_band(int p0, int np, cudaStream_t s, int phase) {
     const int64_t per_pt = (int64_t)n * L;
     const size_t ab_pt = (size_t)geom.ldab * n;
     const size_t nblk = ((size_t)n + geom.nb - 1) / geom.nb;
-    const size_t bp_pt = nblk * 2 * geom.nb, dv_pt = nblk * 2 * geom.nb * geom.nb;
+    const size_t bp_pt = nblk * bp_ints(geom.nb), dv_pt = nblk * 2 * geom.nb * geom.nb;
     // the range's view of the problem: coefficient rows p0 .. p0+np-1
     DevProblem dq = dp;
     dq.N = np;
@@ -1417,7 +1419,7 @@ rsrr_status Handle::sample_band(int p0, int np, cudaStream_t s, int phase) {
         double2 *R = d_R + fo(p0) * per_pt;
         CK(launch_band_lu_r32(ab, piv, info, d_dinvr32 + fo(p0) * dv_pt, geom, np, nn, s, cluster_lu), "band LU");
         if (use_solve2) {
-            CK(launch_block_perm(d_bperm + fo(p0) * bp_pt, piv, nn, geom.kl, geom.nb, np, s), "block permutations");
+            CK(launch_block_perm(d_bperm + fo(p0) * bp_pt, piv, nn, geom.kl, geom.ku, geom.nb, np, s), "block permutations");
             launches += 1;
         }
         if ((ms = mark(2, s)) != RSRR_OK) return ms;
@@ -1440,7 +1442,7 @@ rsrr_status Handle::sample_band(int p0, int np, cudaStream_t s, int phase) {
         double *ab = d_abr64 + fo(p0) * ab_pt, *D = d_Dr64 + fo(p0) * per_pt;
         CK(launch_band_lu_r64(ab, piv, info, d_dinvr64 + fo(p0) * dv_pt, geom, np, nn, s, cluster_lu), "band LU");
         if (use_solve2) {
-            CK(launch_block_perm(d_bperm + fo(p0) * bp_pt, piv, nn, geom.kl, geom.nb, np, s), "block permutations");
+            CK(launch_block_perm(d_bperm + fo(p0) * bp_pt, piv, nn, geom.kl, geom.ku, geom.nb, np, s), "block permutations");
             launches += 1;
         }
         if ((ms = mark(2, s)) != RSRR_OK) return ms;
@@ -1455,7 +1457,7 @@ rsrr_status Handle::sample_band(int p0, int np, cudaStream_t s, int phase) {
         if (phase == 0)
             CK(launch_band_lu_c64(ab, piv, info, d_dinv32 + fo(p0) * dv_pt, geom, np, nn, s, cluster_lu), "band LU");
         if (use_solve2) {
-            CK(launch_block_perm(d_bperm + fo(p0) * bp_pt, piv, nn, geom.kl, geom.nb, np, s), "block permutations");
+            CK(launch_block_perm(d_bperm + fo(p0) * bp_pt, piv, nn, geom.kl, geom.ku, geom.nb, np, s), "block permutations");
             launches += 1;
         }
         if ((ms = mark(2, s)) != RSRR_OK) return ms;
@@ -1482,7 +1484,7 @@ rsrr_status Handle::sample_band(int p0, int np, cudaStream_t s, int phase) {
         if (phase == 0)
             CK(launch_band_lu_c128(ab, piv, info, d_dinv64 + fo(p0) * dv_pt, geom, np, nn, s, cluster_lu), "band LU");
         if (use_solve2) {
-            CK(launch_block_perm(d_bperm + fo(p0) * bp_pt, piv, nn, geom.kl, geom.nb, np, s), "block permutations");
+            CK(launch_block_perm(d_bperm + fo(p0) * bp_pt, piv, nn, geom.kl, geom.ku, geom.nb, np, s), "block permutations");
             launches += 1;
         }
         if ((ms = mark(2, s)) != RSRR_OK) return ms;
@@ -1596,7 +1598,7 @@ rsrr_status Handle::add_points(const cplx *znew, int count, cudaStream_t s) {
             CK(regrow(&d_ab64, ab_pt, N0, N1, false), "regrow band factors");
             CK(regrow(&d_dinv64, nblk * 2 * geom.nb * geom.nb, N0, N1, false), "regrow");
         }
-        if (d_bperm) CK(regrow(&d_bperm, nblk * 2 * geom.nb, N0, N1, false), "regrow");
+        if (d_bperm) CK(regrow(&d_bperm, nblk * bp_ints(geom.nb), N0, N1, false), "regrow");
     }
     if (grow_factors) fcap = N1;
     drop_graph();  // the captured launches name the old buffers

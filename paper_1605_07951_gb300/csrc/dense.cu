@@ -476,7 +476,7 @@ dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_
 // Bound by the FP64 unit (a warp-wide FMA takes 64 cycles of its scheduler, so
 // two FMAs a cycle and SM): what counts is that every SM has work and no lane
 // idles.  One product per point, as before, left 8 blocks on 152 SMs: n = 500,
-// L = 16, 32 points 203 ms for three residuals; all points in one launch 3.4 ms
+// L = 16, 32 points 203 ms for three residuals; all points in one launch 3.1 ms
 // (2.6 ms of FMAs).  The tile is this small so that a few hundred blocks spread
 // evenly.  Sums run over k in order, as the direct path of fp64_gemm's do.
 constexpr int DR_M = 32, DR_N = 16, DR_K = 16, DR_THREADS = 128;

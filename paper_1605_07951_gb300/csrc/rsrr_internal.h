@@ -13,6 +13,9 @@ namespace rsrr {
 // Column block of the band LU and of its solve (they must agree).
 constexpr int NB_C64 = 32;
 constexpr int NB_C128 = 16;
+// Ints of a block's permutation record (band_solve2.cu): 2 nb pairs, their
+// number, the first row above the block; padded to 16 bytes.
+constexpr int bp_ints(int nb) { return 2 * nb + 4; }
 // Largest lower half-bandwidth the band kernels accept (panel rows <= 512).
 constexpr int KL_MAX = 480;
 
@@ -159,19 +162,19 @@ cudaError_t launch_dense_eig_residual(const double2 *V, const double2 *lam, cons
 cudaError_t launch_narrow_all(float2 *D, const double2 *S, int64_t total, cudaStream_t s);
 
 // ---- streaming band solve (band_solve2.cu): composed block permutations
-// (2 nb ints per block) after each LU, then the pipelined solve.  The solve
+// (bp_ints(nb) ints per block) after each LU, then the pipelined solve.  The solve
 // returns cudaErrorInvalidConfiguration when its shared memory (see
 // band_solve2_smem_*) exceeds 227 KB; the caller then uses launch_band_solve_*.
-cudaError_t launch_block_perm(int32_t *bperm, const int32_t *piv, int n, int kl, int nb, int N,
+cudaError_t launch_block_perm(int32_t *bperm, const int32_t *piv, int n, int kl, int ku, int nb, int N,
                               cudaStream_t s);
 size_t band_solve2_smem_c64(const BandGeom &g);
 size_t band_solve2_smem_c128(const BandGeom &g);
-// lc: right-hand sides per CTA, 16 (default), 8, 4 or 2 (more CTAs per point
+// lc: right-hand sides per CTA, 16, 8, 4 or 2, 0 (default): by N and L (more CTAs per point
 // for fewer, the same operations on every column); with gate set, the launch
 // runs only if *gate == want (launch_solve_gate writes it on the device)
 cudaError_t launch_band_solve2_c64(const float2 *ab, const int32_t *bperm, const float2 *dinv,
                                    float2 *B, const BandGeom &g, int N, int n, int L,
-                                   const int32_t *skip, cudaStream_t s, int lc = 16,
+                                   const int32_t *skip, cudaStream_t s, int lc = 0,
                                    const int32_t *gate = nullptr, int want = 0);
 // *gate = k for the narrowest lc = 16 >> k (k = 0..3) whose CTAs for the points
 // with a zero done flag fit in one wave over sms SMs, else 0
