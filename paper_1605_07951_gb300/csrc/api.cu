@@ -665,6 +665,18 @@ rsrr_status prepare(const rsrr_nep *nep, const rsrr_region *region, int32_t N, i
                     delete h;
                     return create_fail("rsrr_create: duplicate entry in the pattern");
                 }
+        // symmetric terms: each column equals its row, in order (rows whose
+        // columns are not sorted count as not symmetric)
+        bool sym = true;
+        for (int64_t c = 0; c < n && sym; ++c) {
+            sym = cptr[c] == h->h_row_ptr[c];
+            for (int32_t q = cptr[c]; q < cptr[c + 1] && sym; ++q) {
+                sym = crow[q] == h->h_col_idx[q];
+                for (size_t t = 0; t < h->fn.size() && sym; ++t)
+                    sym = h->h_vals[t * nnz + q] == h->h_vals[t * nnz + cperm[q]];
+            }
+        }
+        h->sym_real = sym;
         h->h_csc_ptr = std::move(cptr);
         h->h_csc_row = std::move(crow);
         h->h_csc_perm = std::move(cperm);

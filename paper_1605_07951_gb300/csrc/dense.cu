@@ -358,13 +358,26 @@ dense_gemm_update_kernel(C *__restrict__ A_all, int n, int k0) {
 // One CTA per (point, chunk of LC right-hand sides); B (n x L per point,
 // column major) is overwritten with the solution.  Forward per block: the
 // block's interchanges, y = L11^{-1} b_block, rows below -= L21 y.  Backward
-// per block from the end: t = y_block - U12 x_next (columns split across
-// warps, partial tiles summed in shared memory), x = U11^{-1} t.
-constexpr int DS_THREADS = 512;
-constexpr int DS_WARPS = DS_THREADS / 32;
-
-template <typename C, int NB, int LC>
-__global__ void __launch_bounds__(DS_THREADS, 1)
+// per block from the end: x = U11^{-1} y_block, rows above -= U12 x: both
+// updates a thread per row, the factor read along its columns.
+//
+// A block's interchanges are composed by one warp (a lane per pivot: the row
+// at the block's row, and at the row outside that the pivot names first), then
+// applied by all threads at once.
+//
+// IDENT: the right-hand sides are the identity's columns (L = n), B is only
+// written.  A chunk takes the columns whose ones the interchanges bring to LC
+// adjacent rows of one block: its forward pass starts there (two thirds of the
+// forward products are with zeros).
+//
+// FP64 (the inverses of SS-FULL's nodes): bound by the FP64 unit, so lanes must
+// not idle: the backward pass by rows keeps all of them busy where a dot
+// product per row of the block used 16 of 32.  500 matrices of order 233: 78.6
+// -> 35.6 ms.  FP32: bound by reading the factor from L2 once per chunk, so the
+// chunks are as wide as leaves one for every SM: n = 2048, 64 right-hand sides,
+// 32 points 16.8 -> 5.4 ms for three solves.
+template <typename C, int NB, int LC, int TH, bool IDENT>
+__global__ void __launch_bounds__(TH, 512 / TH)
 dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_all,
                    const C *__restrict__ dinv_all, C *__restrict__ B_all, int n, int L,
                    const int32_t *__restrict__ skip) {
@@ -376,94 +389,153 @@ dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_
     const int32_t *piv = piv_all + (size_t)pt * n;
     const int nblk = (n + NB - 1) / NB;
     const C *dinv = dinv_all + (size_t)pt * nblk * 2 * NB * NB;
-    C *B = B_all + (size_t)pt * L * n + (size_t)col0 * n;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    __shared__ C s_D[NB * NB];
-    __shared__ C s_y[NB * LC];
-    __shared__ C s_part[DS_WARPS * NB * LC];
-    // forward
-    for (int k0 = 0; k0 < n; k0 += NB) {
-        const int jb = min(NB, n - k0);
-        for (int q = tid; q < NB * NB; q += DS_THREADS) s_D[q] = dinv[(size_t)(k0 / NB) * 2 * NB * NB + q];
-        if (tid < ncol) {
-            for (int cc = 0; cc < jb; ++cc) {
-                const int p = piv[k0 + cc];
-                if (p != k0 + cc) {
-                    C *a = B + (size_t)tid * n;
-                    const C t = a[k0 + cc]; a[k0 + cc] = a[p]; a[p] = t;
+    C *B = B_all + (size_t)pt * L * n + (IDENT ? 0 : (size_t)col0 * n);
+    const int tid = threadIdx.x;
+    __shared__ __align__(16) C s_D[NB * NB];
+    __shared__ __align__(16) C s_b[NB * LC];
+    __shared__ __align__(16) C s_y[NB * LC];
+    __shared__ int s_col[LC], s_dst[2 * NB], s_src[2 * NB], s_moves;
+    static_assert(!IDENT || NB % LC == 0, "a chunk's ones lie in one block");
+    extern __shared__ int s_perm[];  // IDENT: position -> row, then the pivots
+    if (IDENT) {
+        // the interchanges composed: row s_perm[p] ends at position p
+        for (int i = tid; i < n; i += TH) {
+            s_perm[i] = i;
+            s_perm[n + i] = piv[i];
+        }
+        __syncthreads();
+        if (tid == 0)
+            for (int i = 0; i < n; ++i) {
+                const int p = s_perm[n + i];
+                if (p != i) {
+                    const int t = s_perm[i]; s_perm[i] = s_perm[p]; s_perm[p] = t;
                 }
             }
+        __syncthreads();
+        if (tid < LC) s_col[tid] = tid < ncol ? s_perm[col0 + tid] : 0;
+    } else if (tid < LC) {
+        s_col[tid] = tid;
+    }
+    __syncthreads();
+    size_t cb[LC];  // the columns' places in B
+#pragma unroll
+    for (int c = 0; c < LC; ++c) cb[c] = (size_t)s_col[c] * n;
+    const int k_first = IDENT ? col0 / NB * NB : 0;
+    if (IDENT) {
+        for (int i = tid; i < n; i += TH)
+#pragma unroll
+            for (int c = 0; c < LC; ++c)
+                if (c < ncol) B[cb[c] + i] = i == col0 + c ? cone<C>() : czero<C>();
+        __syncthreads();
+    }
+    // y = D b for the block at k0 (D: its L11^{-1} or U11^{-1}), into s_y and B
+    auto diagonal = [&](int k0, int jb, const C *src) {
+        for (int q = tid; q < NB * NB; q += TH) s_D[q] = src[q];
+        for (int q = tid; q < NB * LC; q += TH) {
+            const int i = q % NB, c = q / NB;
+            s_b[q] = i < jb && c < ncol ? B[(size_t)s_col[c] * n + k0 + i] : czero<C>();
         }
         __syncthreads();
-        for (int q = tid; q < NB * LC; q += DS_THREADS) {
+        for (int q = tid; q < NB * LC; q += TH) {
             const int i = q % NB, c = q / NB;
             C y = czero<C>();
-            if (i < jb && c < ncol) {
-                for (int t = 0; t < jb; ++t) y = cfma(y, s_D[t * NB + i], B[(size_t)c * n + k0 + t]);
-            }
+#pragma unroll 8
+            for (int t = 0; t < NB; ++t) y = cfma(y, s_D[t * NB + i], s_b[c * NB + t]);
             s_y[i * LC + c] = y;
+            if (i < jb && c < ncol) B[(size_t)s_col[c] * n + k0 + i] = y;
         }
         __syncthreads();
-        for (int q = tid; q < jb * LC; q += DS_THREADS) {
-            const int i = q % jb, c = q / jb;
-            if (c < ncol) B[(size_t)c * n + k0 + i] = s_y[i * LC + c];
-        }
-        for (int r = k0 + jb + tid; r < n; r += DS_THREADS) {
+    };
+    // rows r_lo .. r_hi-1 -= A(:, k0 .. k0+jb-1) y
+    auto update = [&](int k0, int jb, int r_lo, int r_hi) {
+        for (int r = r_lo + tid; r < r_hi; r += TH) {
             C acc[LC];
 #pragma unroll
-            for (int c = 0; c < LC; ++c) acc[c] = c < ncol ? B[(size_t)c * n + r] : czero<C>();
-            for (int t = 0; t < jb; ++t) {
-                const C l = A[(int64_t)(k0 + t) * n + r];
+            for (int c = 0; c < LC; ++c) acc[c] = c < ncol ? B[cb[c] + r] : czero<C>();
+            const C *a = A + (size_t)k0 * n + r;
+            if (jb == NB) {
+#pragma unroll 1
+                for (int t0 = 0; t0 < NB; t0 += 8) {
+                    C l[8];
 #pragma unroll
-                for (int c = 0; c < LC; ++c) acc[c] = cfms(acc[c], l, s_y[t * LC + c]);
+                    for (int t = 0; t < 8; ++t) l[t] = a[(size_t)(t0 + t) * n];
+#pragma unroll
+                    for (int t = 0; t < 8; ++t)
+#pragma unroll
+                        for (int c = 0; c < LC; ++c) acc[c] = cfms(acc[c], l[t], s_y[(t0 + t) * LC + c]);
+                }
+            } else {
+                for (int t = 0; t < jb; ++t) {
+                    const C l = a[(size_t)t * n];
+#pragma unroll
+                    for (int c = 0; c < LC; ++c) acc[c] = cfms(acc[c], l, s_y[t * LC + c]);
+                }
             }
 #pragma unroll
             for (int c = 0; c < LC; ++c)
-                if (c < ncol) B[(size_t)c * n + r] = acc[c];
+                if (c < ncol) B[cb[c] + r] = acc[c];
         }
         __syncthreads();
+    };
+    // the interchanges of the block at k0
+    auto interchange = [&](int k0, int jb) {
+        if (tid < 32) {
+            const int lane = tid;
+            const int p = lane < jb ? piv[k0 + lane] : -1;
+            const unsigned same = __match_any_sync(0xffffffffu, p);
+            const bool first = p >= k0 + jb && (same & ((1u << lane) - 1u)) == 0;
+            int top = k0 + lane, out = p;  // rows at block row `lane` and, where first, at row p
+            for (int cc = 0; cc < jb; ++cc) {
+                const int q = __shfl_sync(0xffffffffu, p, cc), a = __shfl_sync(0xffffffffu, top, cc);
+                const unsigned at = __ballot_sync(0xffffffffu, first && p == q);
+                const int b = at ? __shfl_sync(0xffffffffu, out, __ffs(at) - 1) : __shfl_sync(0xffffffffu, top, (q - k0) & 31);
+                if (lane == cc) top = b;
+                if (at) {
+                    if (first && p == q) out = a;
+                } else if (q != k0 + cc && lane == q - k0) {
+                    top = a;
+                }
+            }
+            const bool mt = lane < jb && top != k0 + lane, mo = first && out != p;
+            const unsigned bt = __ballot_sync(0xffffffffu, mt), bo = __ballot_sync(0xffffffffu, mo);
+            const unsigned below = (1u << lane) - 1u;
+            if (mt) {
+                s_dst[__popc(bt & below)] = k0 + lane;
+                s_src[__popc(bt & below)] = top;
+            }
+            if (mo) {
+                s_dst[__popc(bt) + __popc(bo & below)] = p;
+                s_src[__popc(bt) + __popc(bo & below)] = out;
+            }
+            if (lane == 0) s_moves = __popc(bt) + __popc(bo);
+        }
+        __syncthreads();
+        const int items = s_moves * LC;
+        constexpr int PER = (2 * NB * LC + TH - 1) / TH;
+        C v[PER];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const int q = tid + k * TH, e = q / LC, c = q % LC;
+            v[k] = q < items && c < ncol ? B[(size_t)s_col[c] * n + s_src[e]] : czero<C>();
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const int q = tid + k * TH, e = q / LC, c = q % LC;
+            if (q < items && c < ncol) B[(size_t)s_col[c] * n + s_dst[e]] = v[k];
+        }
+        __syncthreads();
+    };
+    for (int k0 = k_first; k0 < n; k0 += NB) {
+        const int jb = min(NB, n - k0);
+        if (!IDENT || k0 > k_first) interchange(k0, jb);
+        diagonal(k0, jb, dinv + (size_t)(k0 / NB) * 2 * NB * NB);
+        update(k0, jb, k0 + jb, n);
     }
-    // backward
     for (int k0 = ((n - 1) / NB) * NB; k0 >= 0; k0 -= NB) {
         const int jb = min(NB, n - k0);
-        const int k1 = k0 + jb;
-        for (int q = tid; q < NB * NB; q += DS_THREADS)
-            s_D[q] = dinv[(size_t)(k0 / NB) * 2 * NB * NB + NB * NB + q];
-        C acc[LC];
-#pragma unroll
-        for (int c = 0; c < LC; ++c) acc[c] = czero<C>();
-        if (lane < jb) {
-            for (int col = k1 + warp; col < n; col += DS_WARPS) {
-                const C u = A[(int64_t)col * n + k0 + lane];
-#pragma unroll
-                for (int c = 0; c < LC; ++c)
-                    if (c < ncol) acc[c] = cfms(acc[c], u, B[(size_t)c * n + col]);
-            }
-        }
-        if (lane < NB) {
-#pragma unroll
-            for (int c = 0; c < LC; ++c) s_part[(warp * NB + lane) * LC + c] = (lane < jb) ? acc[c] : czero<C>();
-        }
-        __syncthreads();
-        for (int q = tid; q < NB * LC; q += DS_THREADS) {
-            const int i = q / LC, c = q % LC;
-            C t = czero<C>();
-            if (i < jb && c < ncol) {
-                t = B[(size_t)c * n + k0 + i];
-                for (int w = 0; w < DS_WARPS; ++w) t = cadd(t, s_part[(w * NB + i) * LC + c]);
-            }
-            s_y[i * LC + c] = t;
-        }
-        __syncthreads();
-        for (int q = tid; q < NB * LC; q += DS_THREADS) {
-            const int i = q / LC, c = q % LC;
-            if (i < jb && c < ncol) {
-                C x = czero<C>();
-                for (int t = 0; t < jb; ++t) x = cfma(x, s_D[t * NB + i], s_y[t * LC + c]);
-                B[(size_t)c * n + k0 + i] = x;
-            }
-        }
-        __syncthreads();
+        diagonal(k0, jb, dinv + (size_t)(k0 / NB) * 2 * NB * NB + NB * NB);
+        update(k0, jb, 0, k0);
     }
 }
 
@@ -736,17 +808,68 @@ cudaError_t launch_dense_lu_c128(double2 *A, int32_t *piv, int32_t *info, double
     return dense_lu_t<double2, NB_C128>(A, piv, info, dinv, n, N, s, launches, nullptr, false);
 }
 
+// chunks of LC right-hand sides: the widest (the factor is read once per chunk)
+// of which there are still enough for the SMs, else the narrowest
+static int ds_columns(int N, int L, int widest) {
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    for (int lc = widest; lc > 4; lc /= 2)
+        if ((int64_t)N * ((L + lc - 1) / lc) >= sms * 4 / 5) return lc;
+    return 4;
+}
+template <typename C, int NB, int LC, int TH>
+static cudaError_t ds_launch(const C *A, const int32_t *piv, const C *dinv, C *B, int n, int N, int L,
+                             const int32_t *skip, cudaStream_t s) {
+    for (int p0 = 0; p0 < N; p0 += 65535) {  // grid.y limit
+        const size_t nblk = ((size_t)n + NB - 1) / NB;
+        dense_solve_kernel<C, NB, LC, TH, false><<<dim3((L + LC - 1) / LC, std::min(N - p0, 65535)), TH, 0, s>>>(
+            A + (size_t)p0 * n * n, piv + (size_t)p0 * n, dinv + p0 * nblk * 2 * NB * NB, B + (size_t)p0 * n * L, n, L,
+            skip ? skip + p0 : nullptr);
+    }
+    return cudaGetLastError();
+}
 cudaError_t launch_dense_solve_c64(const float2 *A, const int32_t *piv, const float2 *dinv, float2 *B,
                                    int n, int N, int L, const int32_t *skip, cudaStream_t s) {
-    dense_solve_kernel<float2, NB_C64, 8><<<dim3((L + 7) / 8, N), DS_THREADS, 0, s>>>(A, piv, dinv, B, n,
-                                                                                      L, skip);
-    return cudaGetLastError();
+    switch (ds_columns(N, L, 16)) {
+    case 16: return ds_launch<float2, NB_C64, 16, 512>(A, piv, dinv, B, n, N, L, skip, s);
+    case 8: return ds_launch<float2, NB_C64, 8, 512>(A, piv, dinv, B, n, N, L, skip, s);
+    default: return ds_launch<float2, NB_C64, 4, 512>(A, piv, dinv, B, n, N, L, skip, s);
+    }
 }
 cudaError_t launch_dense_solve_c128(const double2 *A, const int32_t *piv, const double2 *dinv,
                                     double2 *B, int n, int N, int L, const int32_t *skip,
                                     cudaStream_t s) {
-    dense_solve_kernel<double2, NB_C128, 8><<<dim3((L + 7) / 8, N), DS_THREADS, 0, s>>>(A, piv, dinv, B, n,
-                                                                                       L, skip);
+    if (ds_columns(N, L, 8) == 8) return ds_launch<double2, NB_C128, 8, 256>(A, piv, dinv, B, n, N, L, skip, s);
+    return ds_launch<double2, NB_C128, 4, 256>(A, piv, dinv, B, n, N, L, skip, s);
+}
+// X = (P L U)^{-1}, n x n per point.  The composed interchanges take 2 n ints of
+// shared memory; orders that have no room for them solve with the identity.
+static constexpr int DINV_MAX = 4096;
+__global__ void dense_identity_kernel(double2 *__restrict__ F, int n) {
+    const int64_t nn = (int64_t)n * n;
+    double2 *X = F + (size_t)blockIdx.y * nn;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nn; e += (int64_t)gridDim.x * blockDim.x)
+        X[e] = make_double2(e % n == e / n ? 1.0 : 0.0, 0.0);
+}
+cudaError_t launch_dense_inverse_c128(const double2 *A, const int32_t *piv, const double2 *dinv, double2 *X, int n,
+                                      int N, cudaStream_t s) {
+    constexpr int LC = 8, TH = 256;
+    const size_t nn = (size_t)n * n, nblk = ((size_t)n + NB_C128 - 1) / NB_C128;
+    for (int p0 = 0; p0 < N; p0 += 65535) {  // grid.y limit
+        const int np = std::min(N - p0, 65535);
+        if (n > DINV_MAX) {
+            dense_identity_kernel<<<dim3(grid_for_d((int64_t)nn, 256, 1024), np), 256, 0, s>>>(X + p0 * nn, n);
+            const cudaError_t e = ds_launch<double2, NB_C128, LC, TH>(
+                A + p0 * nn, piv + (size_t)p0 * n, dinv + p0 * nblk * 2 * NB_C128 * NB_C128, X + p0 * nn, n, np, n,
+                nullptr, s);
+            if (e != cudaSuccess) return e;
+            continue;
+        }
+        dense_solve_kernel<double2, NB_C128, LC, TH, true>
+            <<<dim3((n + LC - 1) / LC, np), TH, sizeof(int) * (size_t)(2 * n), s>>>(
+                A + p0 * nn, piv + (size_t)p0 * n, dinv + p0 * nblk * 2 * NB_C128 * NB_C128, X + p0 * nn, n, n,
+                nullptr);
+    }
     return cudaGetLastError();
 }
 

@@ -51,6 +51,7 @@ struct Handle {
     BandGeom geom = {};
     DevProblem dp = {};
     std::vector<std::complex<double>> z;
+    bool sym_real = false;  // sparse kind: every held A_i is symmetric (real values)
     std::vector<int32_t> h_row_ptr, h_col_idx, h_csc_ptr, h_csc_row, h_csc_perm;
     std::vector<double> h_vals;
     // dense problems: the Helmholtz kernel, or caller-supplied dense terms

@@ -150,6 +150,9 @@ cudaError_t launch_dense_solve_c64(const float2 *A, const int32_t *piv, const fl
 cudaError_t launch_dense_solve_c128(const double2 *A, const int32_t *piv, const double2 *dinv,
                                     double2 *B, int n, int N, int L, const int32_t *skip,
                                     cudaStream_t s);
+// X = (P L U)^{-1} (n x n per point) from the factors of launch_dense_lu_c128
+cudaError_t launch_dense_inverse_c128(const double2 *A, const int32_t *piv, const double2 *dinv, double2 *X, int n,
+                                      int N, cudaStream_t s);
 cudaError_t launch_dense_residual(double2 *R, const double2 *T, const double2 *X, const double2 *U, int n, int L,
                                   int N, const int32_t *done, cudaStream_t s);
 cudaError_t launch_dense_colmax(const double2 *R, const double2 *X, int n, int L, int N, double *rmax,

@@ -8,9 +8,11 @@
 // (Section 5.1) and scaled powers s_q = (z_q - gamma) / rho, rho = max(a, b).
 // Nodes are processed in chunks: T_Q(z_q) = sum_i f_i(z_q) P_i is assembled
 // for every node of the chunk, factored by the batched complex128 dense LU
-// (partial pivoting), T_Q^{-1} obtained by the batched solve with the identity
-// as right-hand side, and the weighted inverses summed into the moments in a
-// fixed node order.  The Hankel SVD and the small eigenproblem stay on the
+// (partial pivoting), inverted, and the weighted inverses summed into the
+// moments in a fixed node order.  For symmetric real A_i and f_i with
+// f_i(conj z) = conj f_i(z), T_Q(conj z) = T_Q(z)^H: on a contour symmetric
+// about the real axis only one node of each conjugate pair is factored, half
+// of the work (bound by the FP64 unit).  The Hankel SVD and the small eigenproblem stay on the
 // host (ssfull_host.cpp).
 #include <algorithm>
 #include <cmath>
@@ -34,25 +36,43 @@ __global__ void tq_assemble_kernel(double2 *__restrict__ T, const double2 *__res
     }
 }
 
-// F[b] = I (k x k) for every node of a chunk
-__global__ void tq_identity_kernel(double2 *__restrict__ F, int k) {
-    const int b = blockIdx.y;
-    const int64_t kk = (int64_t)k * k;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < kk;
-         e += (int64_t)gridDim.x * blockDim.x)
-        F[(size_t)b * kk + e] = make_double2(e % k == e / k ? 1.0 : 0.0, 0.0);
-}
-
-// Acc[alpha] += sum_b c[b][alpha] F[b], nodes summed in order
-__global__ void tq_moment_kernel(double2 *__restrict__ Acc, const double2 *__restrict__ F,
-                                 const double2 *__restrict__ c, int nb, int nmom, int64_t kk) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < kk;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        for (int al = 0; al < nmom; ++al) {
-            double2 acc = Acc[(size_t)al * kk + e];
-            for (int b = 0; b < nb; ++b) acc = cfma(acc, c[(size_t)b * nmom + al], F[(size_t)b * kk + e]);
-            Acc[(size_t)al * kk + e] = acc;
+// Acc[alpha] += sum_b c[b][alpha] F[b] + d[b][alpha] F[b]^H, nodes summed in
+// order.  A block of 256 threads owns a 16 x 16 tile; the mirrored tile it needs
+// for F^H comes through shared memory (mirror = 0: d is zero and not read).
+__global__ void __launch_bounds__(256)
+tq_moment_kernel(double2 *__restrict__ Acc, const double2 *__restrict__ F, const double2 *__restrict__ c,
+                 const double2 *__restrict__ d, int nb, int nmom, int k, int mirror) {
+    __shared__ double2 s_t[16][17];
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    const int i = blockIdx.x * 16 + tx, j = blockIdx.y * 16 + ty;        // this thread's element
+    const int mi = blockIdx.y * 16 + tx, mj = blockIdx.x * 16 + ty;      // its part of the mirrored tile
+    const bool in = i < k && j < k, min = mi < k && mj < k;
+    const size_t kk = (size_t)k * k, e = (size_t)j * k + i, me = (size_t)mj * k + mi;
+    for (int al0 = 0; al0 < nmom; al0 += 4) {
+        double2 acc[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            acc[a] = in && al0 + a < nmom ? Acc[(al0 + a) * kk + e] : make_double2(0.0, 0.0);
+        for (int b = 0; b < nb; ++b) {
+            const double2 f = in ? F[b * kk + e] : make_double2(0.0, 0.0);
+            double2 h = make_double2(0.0, 0.0);
+            if (mirror) {
+                __syncthreads();
+                s_t[ty][tx] = min ? F[b * kk + me] : make_double2(0.0, 0.0);
+                __syncthreads();
+                h = s_t[tx][ty];
+                h.y = -h.y;
+            }
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                if (al0 + a >= nmom) break;
+                acc[a] = cfma(acc[a], c[(size_t)b * nmom + al0 + a], f);
+                if (mirror) acc[a] = cfma(acc[a], d[(size_t)b * nmom + al0 + a], h);
+            }
         }
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            if (in && al0 + a < nmom) Acc[(al0 + a) * kk + e] = acc[a];
     }
 }
 
@@ -71,9 +91,9 @@ size_t ssfull_dev_bytes(int64_t k, int m, int NQ, int KQ) {
     const size_t B = ssfull_chunk(k, NQ, kSsfullChunkBytes);
     const size_t kk = (size_t)k * k;
     const size_t nblk = ((size_t)k + NB_C128 - 1) / NB_C128;
-    return sizeof(double2) * (2 * B * kk + (size_t)2 * KQ * kk + B * (m + 2 * KQ) +
+    return sizeof(double2) * (2 * B * kk + (size_t)2 * KQ * kk + B * (m + 4 * KQ) +
                               B * nblk * 2 * NB_C128 * NB_C128) +
-           sizeof(int32_t) * (B * k + B) + 8 * 256;
+           sizeof(int32_t) * (B * k + B) + 9 * 256;
 }
 
 rsrr_status Handle::ssfull_moments(const std::vector<std::complex<double>> &fq,
@@ -107,6 +127,7 @@ rsrr_status Handle::ssfull_moments(const std::vector<std::complex<double>> &fq,
     double2 *dA = reinterpret_cast<double2 *>(take(sizeof(double2) * nmom * kk));
     double2 *df = reinterpret_cast<double2 *>(take(sizeof(double2) * B * m));
     double2 *dc = reinterpret_cast<double2 *>(take(sizeof(double2) * B * nmom));
+    double2 *dd = reinterpret_cast<double2 *>(take(sizeof(double2) * B * nmom));
     double2 *dinv = reinterpret_cast<double2 *>(take(sizeof(double2) * B * nblk * 2 * NB_C128 * NB_C128));
     int32_t *dpiv = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * B * k));
     int32_t *dinfo = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * B));
@@ -114,46 +135,62 @@ rsrr_status Handle::ssfull_moments(const std::vector<std::complex<double>> &fq,
 
     const double rho = std::max(region.a, region.b);
     const cplx gamma(region.center.re, region.center.im);
-    std::vector<double2> hf((size_t)B * m), hc((size_t)B * nmom);
+    // nodes to factor: all, or one of each conjugate pair (q, NQ - 1 - q); the
+    // pair's values agree to rounding or the symmetry is not used
+    bool paired = sym_real;
+    auto conj_close = [](cplx a, cplx b) { return std::abs(a - std::conj(b)) <= 16.0 * 2.2204460492503131e-16 * std::abs(b); };
+    for (int q = 0; q < NQ && paired; ++q) {
+        const int r = NQ - 1 - q;
+        paired = conj_close(zq[r], zq[q]);
+        for (int i = 0; i < m && paired; ++i) paired = conj_close(fq[(size_t)r * m + i], fq[(size_t)q * m + i]);
+    }
+    const int nodes = paired ? (NQ + 1) / 2 : NQ;
+    std::vector<double2> hf((size_t)B * m), hc((size_t)B * nmom), hd((size_t)B * nmom);
     std::vector<int32_t> info(B);
     if ((e = cudaMemsetAsync(dA, 0, sizeof(double2) * nmom * kk, s)) != cudaSuccess)
         return fail(RSRR_ECUDA, "memset", e);
-    for (int q0 = 0; q0 < NQ; q0 += B) {
-        const int nb = std::min(B, NQ - q0);
+    for (int q0 = 0; q0 < nodes; q0 += B) {
+        const int nb = std::min(B, nodes - q0);
         for (int bq = 0; bq < nb; ++bq) {
             const int q = q0 + bq;
-            const cplx z = zq[q], w = wq[q];
             for (int i = 0; i < m; ++i) {
                 const cplx v = fq[(size_t)q * m + i];
                 hf[(size_t)bq * m + i] = make_double2(v.real(), v.imag());
             }
-            const cplx sz = (z - gamma) / rho;
-            cplx c = w;
-            for (int al = 0; al < nmom; ++al) {
-                hc[(size_t)bq * nmom + al] = make_double2(c.real(), c.imag());
-                c *= sz;
-            }
+            auto powers = [&](int node, std::vector<double2> &out) {
+                const cplx sz = (zq[node] - gamma) / rho;
+                cplx c = wq[node];
+                for (int al = 0; al < nmom; ++al) {
+                    out[(size_t)bq * nmom + al] = make_double2(c.real(), c.imag());
+                    c *= sz;
+                }
+            };
+            powers(q, hc);
+            if (paired && NQ - 1 - q != q) powers(NQ - 1 - q, hd);
+            else std::fill(hd.begin() + (size_t)bq * nmom, hd.begin() + (size_t)(bq + 1) * nmom, make_double2(0.0, 0.0));
         }
-        // (pageable sources: each copy returns once staged, so hf/hc may be refilled)
+        // (pageable sources: each copy returns once staged, so hf, hc, hd may be refilled)
         if ((e = cudaMemcpyAsync(df, hf.data(), sizeof(double2) * nb * m, cudaMemcpyHostToDevice, s)) !=
                 cudaSuccess ||
             (e = cudaMemcpyAsync(dc, hc.data(), sizeof(double2) * nb * nmom, cudaMemcpyHostToDevice, s)) !=
+                cudaSuccess ||
+            (e = cudaMemcpyAsync(dd, hd.data(), sizeof(double2) * nb * nmom, cudaMemcpyHostToDevice, s)) !=
                 cudaSuccess)
             return fail(RSRR_ECUDA, "SS-FULL coefficients", e);
         tq_assemble_kernel<<<dim3(grid_cap(kk, 256, 1024), nb), 256, 0, s>>>(dT, d_P, df, m, kk);
-        tq_identity_kernel<<<dim3(grid_cap(kk, 256, 1024), nb), 256, 0, s>>>(dF, k);
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(RSRR_ECUDA, "SS-FULL assemble", e);
         if ((e = launch_dense_lu_c128(dT, dpiv, dinfo, dinv, k, nb, s, &launches)) != cudaSuccess)
             return fail(RSRR_ECUDA, "SS-FULL LU", e);
-        if ((e = launch_dense_solve_c128(dT, dpiv, dinv, dF, k, nb, k, nullptr, s)) != cudaSuccess)
+        if ((e = launch_dense_inverse_c128(dT, dpiv, dinv, dF, k, nb, s)) != cudaSuccess)
             return fail(RSRR_ECUDA, "SS-FULL inverse", e);
-        tq_moment_kernel<<<grid_cap(kk, 256, 152 * 8), 256, 0, s>>>(dA, dF, dc, nb, nmom, kk);
+        const unsigned tiles = (unsigned)((k + 15) / 16);
+        tq_moment_kernel<<<dim3(tiles, tiles), 256, 0, s>>>(dA, dF, dc, dd, nb, nmom, k, paired ? 1 : 0);
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(RSRR_ECUDA, "SS-FULL moments", e);
         if ((e = cudaMemcpyAsync(info.data(), dinfo, sizeof(int32_t) * nb, cudaMemcpyDeviceToHost, s)) !=
                 cudaSuccess ||
             (e = cudaStreamSynchronize(s)) != cudaSuccess)
             return fail(RSRR_ECUDA, "SS-FULL chunk", e);
-        launches += 4;
+        launches += 3;
         for (int bq = 0; bq < nb; ++bq)
             if (info[bq] != 0)
                 return fail(RSRR_ESINGULAR, "rsrr_solve: projected T_Q singular at a quadrature node");
