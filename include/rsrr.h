@@ -557,7 +557,9 @@ rsrr_status rsrr_solve_band_noalloc(int64_t n, int32_t kl, int32_t ku, const rsr
  *   max_ws_bytes  0: work space for the whole product; else its upper bound
  *              (the product then runs in chunks of K)
  *   stream     work is queued on it; the call waits for it before returning
- * Work space is allocated and freed inside the call.  Returns OK, EINVAL,
+ * Work space comes from a pool of the library, which keeps at most 2 GiB of it
+ * on the device between calls and gives that back when a handle or a server is
+ * created; it does not survive a cudaDeviceReset.  Returns OK, EINVAL,
  * ENOMEM (work space), ETIMEOUT (a bounded wait of the tensor-core kernel ran
  * out) or ECUDA; the message is in rsrr_last_error(NULL). */
 rsrr_status rsrr_zgemm(int32_t M, int32_t N, int32_t K, int32_t conjA, const rsrr_c128 *A,

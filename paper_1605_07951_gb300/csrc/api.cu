@@ -380,6 +380,7 @@ rsrr_status rsrr_create(const rsrr_nep *nep, const rsrr_region *region, int32_t 
     Handle *h = nullptr;
     rsrr_status st = rsrr::prepare(nep, region, N, L, opts, &h);
     if (st != RSRR_OK) return st;
+    rsrr::zgemm_release_kept();
     if (h->opts.mem_budget_bytes > 0) {
         size_t need = h->estimate_bytes();
         const size_t budget = (size_t)h->opts.mem_budget_bytes;

@@ -24,14 +24,15 @@
 //    FP32 sum; the tensor cores round such mixed-magnitude sums (measured:
 //    a shared group-4..6 accumulator lost ~0.3 units of 2^-46), which at
 //    this weight stays below 2^-54.  Pairs with t >= 7 (below 2^-56
-//    relative) are dropped.  At most 512 folds per product keep |acc| below
-//    2^62 (K is chunked beyond 32768).
+//    relative) are dropped.  |acc| stays below K' 2^46 (every |x| < 1), so
+//    K' <= 98304 keeps it below 2^62.6 (K is chunked beyond 49152).
 // 4. C~_ij = 2^(e_i + f_j) 2^-46 (acc + 2^32 low), rounded once to FP64.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <mutex>
 #include <string>
 
 #include "rsrr.h"
@@ -49,7 +50,7 @@ constexpr int OZ_LD = OZ_KC + 8;  // shared-memory row length (bf16): 80 bytes, 
 constexpr int OZ_NS = 3;          // pipeline stages
 constexpr int OZ_FOLD = 4;        // stages per exact fold (K' = 128)
 constexpr int OZ_BCACHE = 4;      // B slices held in registers per 16-deep step
-constexpr int64_t OZ_KMAX = 32768;  // complex K per chunk: <= 512 folds
+constexpr int64_t OZ_KMAX = 49152;  // complex K per chunk: K' 2^46 < 2^63, the 64-bit sums do not overflow
 constexpr int OZ_THREADS = 256;   // 8 warps: 2 (M) x 4 (N), 32 x 16 outputs each
 constexpr int OZ_ROWS = OZ_S * (OZ_BM + OZ_BN);         // shared-memory rows per stage
 constexpr int OZ_STAGE = OZ_ROWS * OZ_LD;                // bf16 elements per stage
@@ -92,9 +93,9 @@ RSRR_DEV void digits7(long long m, float out[OZ_S]) {
 
 // ----------------------------------------------------------- exponents
 // E[c] = largest biased exponent in column c (contiguous, K entries); also
-// written to E[c + dup] when dup > 0 (the Im-output columns of B~)
+// written to E[c + dup] when dup > 0 (the Im-output columns of B~) and to E2[c]
 __global__ void oz_colexp_kernel(int *__restrict__ E, const double2 *__restrict__ X, int64_t ld,
-                                 int K, int cols, int dup) {
+                                 int K, int cols, int dup, int *__restrict__ E2) {
     __shared__ int w[32];
     for (int c = blockIdx.x; c < cols; c += gridDim.x) {
         int m = 1;
@@ -110,6 +111,7 @@ __global__ void oz_colexp_kernel(int *__restrict__ E, const double2 *__restrict_
             for (int q = 0; q < (int)(blockDim.x >> 5); ++q) r = max(r, w[q]);
             E[c] = r;
             if (dup > 0) E[c + dup] = r;
+            if (E2) E2[c] = r;
         }
         __syncthreads();
     }
@@ -156,25 +158,25 @@ RSRR_DEV void store_zero(__nv_bfloat16 *P, size_t stride, size_t off) {
 
 // Rows built from contiguous columns of X.
 //   mode 0 (A^H):  row r = conj(column r),                  r < R
-//   mode 1 (B):    row r < Nc: (Re, -Im) of column r;  Nc <= r < 2Nc: (Im, Re) of column r - Nc
-// Rows >= R and k >= K are written as zeros.
+//   mode 1 (B):    row r < H: (Re, -Im) of column r;  H <= r < 2H: (Im, Re) of column r - H
+// Rows of columns >= R and k >= K are written as zeros.
 __global__ void oz_slice_cols_kernel(__nv_bfloat16 *__restrict__ P, const int *__restrict__ E,
                                      const double2 *__restrict__ X, int64_t ld, int mode, int R,
-                                     int Nc, int K, int Rp, int Kp) {
+                                     int H, int K, int Rp, int Kp) {
     const size_t stride = (size_t)Rp * Kp;
     const int Kh = Kp / 2;
     for (int r = blockIdx.y; r < Rp; r += gridDim.y) {
-        const int c = (mode == 1 && r >= Nc) ? r - Nc : r;
-        const int Ec = (r < R) ? E[c] : 1;
+        const int c = (mode == 1 && r >= H) ? r - H : r;
+        const int Ec = (c < R) ? E[c] : 1;
         for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Kh; k += gridDim.x * blockDim.x) {
             const size_t off = (size_t)r * Kp + 2 * (size_t)k;
-            if (r >= R || k >= K) {
+            if (c >= R || k >= K) {
                 store_zero(P, stride, off);
                 continue;
             }
             const double2 v = X[(int64_t)c * ld + k];
             double re = v.x, im = -v.y;
-            if (mode == 1 && r >= Nc) { re = v.y; im = v.x; }
+            if (mode == 1 && r >= H) { re = v.y; im = v.x; }
             store_slices(P, stride, off, re, im, Ec);
         }
     }
@@ -217,42 +219,74 @@ __global__ void oz_slice_rows_kernel(__nv_bfloat16 *__restrict__ P, const int *_
 //   per-slice operand (A):          ss = 16 TR,  kcs = 8 TR
 //   slices stacked per core column (B, read as one N = 64 q operand):
 //                                   ss = 8 TR,   kcs = 8 OZ_S TR
-// Rows as in oz_slice_cols_kernel (mode 0, 1) or rows of the column-major X
-// itself (mode 2, as oz_slice_rows_kernel); rows >= R and k >= K are zeros.
 // One warp per 8 rows x 4 complex K (a core matrix of every slice): lane =
 // 4 (row % 8) + k % 4, so every slice store of a warp is 128 contiguous bytes.
-__global__ void oz_slice_tiled_kernel(__nv_bfloat16 *__restrict__ P, const int *__restrict__ E,
-                                      const double2 *__restrict__ X, int64_t ld, int mode, int R,
-                                      int Nc, int K, int Rp, int Kp, int TR, int stacked) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nrg = Rp / 8, nkg = Kp / 8, total = nrg * nkg;
-    const int64_t nks = Kp / 16;
-    const size_t ss = stacked ? 8 * (size_t)TR : 16 * (size_t)TR;
+RSRR_DEV size_t tiled_offset(int r, int64_t kg, int lane, int64_t nks, int TR, bool stacked) {
     const size_t kcs = stacked ? 8 * (size_t)OZ_S * TR : 8 * (size_t)TR;
     const size_t chunk = (size_t)OZ_S * TR * 16;
+    return ((size_t)(r / TR) * nks + (size_t)(kg >> 1)) * chunk + (size_t)(kg & 1) * kcs + 8 * (size_t)(r % TR) +
+           2 * (lane & 3);
+}
+RSRR_DEV void store_digits(__nv_bfloat16 *P, size_t stride, size_t off, const float (&re)[OZ_S], const float (&im)[OZ_S]) {
+#pragma unroll
+    for (int s = 0; s < OZ_S; ++s)
+        *reinterpret_cast<__nv_bfloat162 *>(P + s * stride + off) = __floats2bfloat162_rn(re[s], im[s]);
+}
+
+// The columns of X as rows: (Re, -Im) of column c to row c of PA (A^H, RA rows;
+// may be null) and of PB, (Im, Re) to row H + c of PB (may be null).  Columns
+// >= R and k >= K are zeros.  One pass serves both halves of B~ and, for a
+// Hermitian product, A~ too: X is read and digitised once instead of three times.
+__global__ void oz_slice_columns_kernel(__nv_bfloat16 *__restrict__ PA, int RA, __nv_bfloat16 *__restrict__ PB, int H,
+                                        int Np, const int *__restrict__ E, const double2 *__restrict__ X, int64_t ld,
+                                        int R, int K, int Kp, int TA, int TB) {
+    const int lane = threadIdx.x & 31;
+    const int rows = max(PA ? RA : 0, PB ? max(H, Np - 2 * H) : 0);
+    const int64_t nkg = Kp / 8, total = (int64_t)((rows + 7) / 8) * nkg, nks = Kp / 16;
     const int64_t wstep = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += wstep) {
-        // consecutive warps along the contiguous direction of X
-        const int64_t rg = mode == 2 ? w % nrg : w / nkg;
-        const int64_t kg = mode == 2 ? w / nrg : w % nkg;
-        const int r = (int)(8 * rg) + (lane >> 2);
-        const int k = (int)(4 * kg) + (lane & 3);  // complex index, k' = 2k
-        const size_t off = ((size_t)(r / TR) * nks + (size_t)(kg >> 1)) * chunk + (size_t)(kg & 1) * kcs +
-                           8 * (size_t)(r % TR) + 2 * (lane & 3);
+        const int64_t kg = w % nkg;  // consecutive warps along the columns
+        const int c = (int)(8 * (w / nkg)) + (lane >> 2), k = (int)(4 * kg) + (lane & 3);
+        float re[OZ_S], im[OZ_S], nim[OZ_S];
+        double2 v = make_double2(0.0, 0.0);
+        int e = 1;
+        if (c < R && k < K) {
+            v = X[(int64_t)c * ld + k];
+            e = E[c];
+        }
+        digits7(fixed55(v.x, e), re);
+        digits7(fixed55(-v.y, e), nim);
+        if (PA && c < RA) store_digits(PA, 16 * (size_t)TA, tiled_offset(c, kg, lane, nks, TA, false), re, nim);
+        if (PB && c < H) {
+            digits7(fixed55(v.y, e), im);
+            store_digits(PB, 8 * (size_t)TB, tiled_offset(c, kg, lane, nks, TB, true), re, nim);
+            store_digits(PB, 8 * (size_t)TB, tiled_offset(H + c, kg, lane, nks, TB, true), im, re);
+        }
+        // rows of the last tile past the second half
+        if (PB && c + 2 * H < Np) {
+            const float z[OZ_S] = {};
+            store_digits(PB, 8 * (size_t)TB, tiled_offset(c + 2 * H, kg, lane, nks, TB, true), z, z);
+        }
+    }
+}
+
+// Rows of the column-major X itself (A); rows >= R and k >= K are zeros.
+__global__ void oz_slice_rows_tiled_kernel(__nv_bfloat16 *__restrict__ P, const int *__restrict__ E,
+                                           const double2 *__restrict__ X, int64_t ld, int R, int K, int Rp, int Kp,
+                                           int TR) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nrg = Rp / 8, total = nrg * (Kp / 8), nks = Kp / 16;
+    const int64_t wstep = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += wstep) {
+        const int64_t rg = w % nrg, kg = w / nrg;  // consecutive warps along the rows
+        const int r = (int)(8 * rg) + (lane >> 2), k = (int)(4 * kg) + (lane & 3);
+        const size_t off = tiled_offset(r, kg, lane, nks, TR, false);
         if (r >= R || k >= K) {
-            store_zero(P, ss, off);
+            store_zero(P, 16 * (size_t)TR, off);
             continue;
         }
-        if (mode == 2) {
-            const double2 v = X[(int64_t)k * ld + r];
-            store_slices(P, ss, off, v.x, v.y, E[r]);
-        } else {
-            const int c = (mode == 1 && r >= Nc) ? r - Nc : r;
-            const double2 v = X[(int64_t)c * ld + k];
-            double re = v.x, im = -v.y;
-            if (mode == 1 && r >= Nc) { re = v.y; im = v.x; }
-            store_slices(P, ss, off, re, im, E[c]);
-        }
+        const double2 v = X[(int64_t)k * ld + r];
+        store_slices(P, 16 * (size_t)TR, off, v.x, v.y, E[r]);
     }
 }
 
@@ -294,6 +328,17 @@ RSRR_DEV long long scaled_group_to_ll(float f) {
     return bits < 0 ? -m : m;
 }
 
+// 2^n (acc + 2^32 low), rounded once to FP64 in the sum.  The exponent is added
+// in integers: the FP64 unit, whose instructions take 64 cycles a warp, is left
+// with the two conversions and one FMA.
+RSRR_DEV double oz_value(long long acc, float low, int n) {
+    const double d = fma((double)low, 0x1p32, (double)acc);
+    const long long b = __double_as_longlong(d);
+    const int ex = (int)((b >> 52) & 0x7FF), nx = ex + n;
+    if (ex >= 1 && ex <= 2046 && nx >= 1 && nx <= 2046) return __longlong_as_double(b + ((long long)n << 52));
+    return ldexp(d, n);
+}
+
 // One CTA: a 64 x 64 tile of C~ over K' range [sp kchunk, (sp+1) kchunk).
 // W != null: FP64 partial tile into W[sp][i][j'] (Mp x Np, row major).
 // W == null: C = alpha C~ + beta C written directly (one split).
@@ -301,7 +346,7 @@ RSRR_DEV long long scaled_group_to_ll(float f) {
 __global__ void __launch_bounds__(OZ_THREADS, 1)
 oz_gemm_kernel(const __nv_bfloat16 *__restrict__ As, const __nv_bfloat16 *__restrict__ Bs,
                const int *__restrict__ Ea, const int *__restrict__ Eb, double *__restrict__ W,
-               double2 *__restrict__ C, int64_t ldc, int M, int N, int Mp, int Np, int Kp, int kchunk,
+               double2 *__restrict__ C, int64_t ldc, int M, int N, int H, int Mp, int Np, int Kp, int kchunk,
                int halfN_tiles, int upper_only, double alpha, double beta) {
     const int bm = blockIdx.x, bn = blockIdx.y, sp = blockIdx.z;
     if (upper_only && bm > (bn % halfN_tiles)) return;
@@ -421,12 +466,11 @@ oz_gemm_kernel(const __nv_bfloat16 *__restrict__ As, const __nv_bfloat16 *__rest
             for (int q = 0; q < 4; ++q) {
                 const int i = m0 + wm * 32 + a * 16 + g + (q >= 2 ? 8 : 0);
                 const int jj = n0 + wn * 16 + b * 8 + 2 * tq + (q & 1);
-                const double v = ldexp((double)acc[a][b][q] + (double)low[a][b][q] * 0x1p32,
-                                       Ea[i] + Eb[jj] - 2090);
+                const double v = oz_value(acc[a][b][q], low[a][b][q], Ea[i] + Eb[jj] - 2090);
+                const int part = jj >= H, j = jj - part * H;
                 if (W) {
                     W[(size_t)sp * Mp * Np + (size_t)i * Np + jj] = v;
-                } else if (i < M && jj < 2 * N) {
-                    const int part = jj >= N, j = jj - part * N;
+                } else if (i < M && j < N) {
                     double *c = reinterpret_cast<double *>(C + (int64_t)j * ldc + i) + part;
                     double r = alpha * v;
                     if (beta != 0.0) r = fma(beta, *c, r);
@@ -439,7 +483,7 @@ oz_gemm_kernel(const __nv_bfloat16 *__restrict__ As, const __nv_bfloat16 *__rest
 // The same products on the 5th-generation tensor cores: a CTA of 256 threads
 // owns a 128 x 64 tile of C~.  Per 16-deep stage of K' the 7 A slices (128
 // rows) and the 7 B slices (64 rows each, stacked to 448 rows) arrive by two
-// bulk copies of the TMA engine (the stage images of oz_slice_tiled_kernel,
+// bulk copies of the TMA engine (the stage images of the slicing kernels,
 // 28 and 14 KB, contiguous in global memory; issued by one thread, completion
 // counted in bytes on the stage's mbarrier) in the K-major core-matrix layout
 // (8 rows x 16 bytes per core matrix, no swizzle), in a ring of OZT_NST
@@ -465,6 +509,7 @@ constexpr int OZT_BN = 64;
 constexpr int OZT_KC = 16;
 constexpr int OZT_THREADS = 512;                 // 16 warps: 4 lane quarters x 4 column groups
 constexpr int OZT_CPT = OZT_BN / (OZT_THREADS / 128);  // tile columns a thread folds (16)
+constexpr int OZT_GM = 8;                        // row tiles of a group (order of the tiles)
 constexpr int OZT_PRODUCER = OZT_THREADS / 2;    // the copy thread (first lane of the upper half)
 constexpr int OZT_A_SLICE = OZT_BM * OZT_KC * 2;           // bytes of one A slice per stage
 constexpr int OZT_B_SLICE = OZT_BN * OZT_KC * 2;           // bytes of one B slice per stage
@@ -568,10 +613,17 @@ RSRR_DEV int group_int(float g, float s12, float s) {
 __global__ void __launch_bounds__(OZT_THREADS, 1)
 oz_gemm_tc_kernel(const __nv_bfloat16 *__restrict__ As, const __nv_bfloat16 *__restrict__ Bs,
                   const int *__restrict__ Ea, const int *__restrict__ Eb, double *__restrict__ W,
-                  double2 *__restrict__ C, int64_t ldc, int M, int N, int Mp, int Np, int Kp, int kchunk,
+                  double2 *__restrict__ C, int64_t ldc, int M, int N, int H, int Mp, int Np, int Kp, int kchunk,
                   int halfN_tiles, int upper_only, double alpha, double beta,
                   unsigned int *__restrict__ status) {
-    const int bm = blockIdx.x, bn = blockIdx.y, sp = blockIdx.z;
+    // tiles in groups of OZT_GM row tiles by all column tiles, row tiles first: the
+    // CTAs at work together share few stage images of either operand, which
+    // then come from L2 (column by column of tiles, a tall product read its
+    // A~ from DRAM once per column: 40000 x 237 x 237 909 -> GEMM_US us)
+    const int nbm = Mp / OZT_BM, nbn = Np / OZT_BN;
+    const int grp = blockIdx.x / (OZT_GM * nbn), in = blockIdx.x % (OZT_GM * nbn);
+    const int gm = min(OZT_GM, nbm - grp * OZT_GM);  // the last group may be narrower
+    const int bm = grp * OZT_GM + in % gm, bn = in / gm, sp = blockIdx.z;
     if (upper_only && OZT_BM * bm > OZT_BN * (bn % halfN_tiles) + OZT_BN - 1) return;
     extern __shared__ __align__(1024) unsigned char ozt_smem[];
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(ozt_smem);
@@ -727,13 +779,13 @@ oz_gemm_tc_kernel(const __nv_bfloat16 *__restrict__ As, const __nv_bfloat16 *__r
 #pragma unroll
     for (int c = 0; c < OZT_CPT; ++c) {
         const int jj = n0 + lcol + c;
-        const double v = ldexp((double)acc[c] + (double)low[c] * 0x1p32, ea + Eb[jj] - 2090);
+        const double v = oz_value(acc[c], low[c], ea + Eb[jj] - 2090);
+        const int part = jj >= H, j = jj - part * H;
         if (W) {
             W[(size_t)sp * Mp * Np + (size_t)i * Np + jj] = v;
-        } else if (i < M && jj < 2 * N) {
-            const int part = jj >= N, j = jj - part * N;
+        } else if (i < M && j < N) {
             double *cp = reinterpret_cast<double *>(C + (int64_t)j * ldc + i) + part;
-            double r = alpha * v;
+            double r = alpha == 1.0 ? v : alpha * v;
             if (beta != 0.0) r = fma(beta, *cp, r);
             *cp = r;
         }
@@ -761,7 +813,7 @@ cudaError_t launch_wait_check(long long limit, unsigned int *status, cudaStream_
 
 // C = alpha sum_s W[s] + beta C (fixed order over the splits)
 __global__ void oz_combine_kernel(double2 *__restrict__ C, int64_t ldc, const double *__restrict__ W,
-                                  int M, int N, int Mp, int Np, int splits, double alpha, double beta,
+                                  int M, int N, int H, int Mp, int Np, int splits, double alpha, double beta,
                                   int upper_only, int bm) {
     const int64_t total = (int64_t)M * N;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
@@ -772,7 +824,7 @@ __global__ void oz_combine_kernel(double2 *__restrict__ C, int64_t ldc, const do
         for (int s = 0; s < splits; ++s) {
             const double *Wp = W + (size_t)s * Mp * Np + (size_t)i * Np;
             re += Wp[j];
-            im += Wp[N + j];
+            im += Wp[H + j];
         }
         double2 r = make_double2(alpha * re, alpha * im);
         if (beta != 0.0) {
@@ -818,6 +870,7 @@ static int grid_for(int64_t work) {
 namespace {
 struct OzPlan {
     int64_t Mp, Np, Kc, Kp;  // Kc: complex K per chunk
+    int64_t H;               // first column of C~ that holds imaginary parts
     int splits;
     int64_t kchunk;          // K' per split
     size_t bytes;
@@ -857,11 +910,14 @@ int64_t tile_count(int64_t Mp, int64_t Np, int bm, bool upper, int64_t halfN) {
     return t;
 }
 
-OzPlan make_plan(int M, int N, int K, bool hermitian, size_t ws_bytes, int bm) {
+OzPlan make_plan(int M, int N, int K, bool hermitian, size_t ws_bytes, int bm, int64_t kmax = OZ_KMAX) {
     OzPlan p{};
     p.Mp = rup(M, bm);
-    p.Np = rup(2 * (int64_t)N, OZ_BN);
-    const int64_t tiles = (p.Mp / bm) * (p.Np / OZ_BN) / (hermitian ? 2 : 1);
+    // a Hermitian result's halves start on tiles of their own, so that the tiles
+    // below the diagonal of both can be left out
+    p.H = hermitian ? rup(N, OZ_BN) : N;
+    p.Np = rup(2 * p.H, OZ_BN);
+    const int64_t tiles = tile_count(p.Mp, p.Np, bm, hermitian, hermitian ? p.H / OZ_BN : p.Np / OZ_BN);
     const int64_t Kall = std::max(K, 1);
     auto fit = [&](int64_t kc) {
         p.Kc = kc;
@@ -871,29 +927,28 @@ OzPlan make_plan(int M, int N, int K, bool hermitian, size_t ws_bytes, int bm) {
         p.bytes = plan_bytes(p.Mp, p.Np, p.Kp, p.splits);
         return p.bytes <= ws_bytes;
     };
-    int64_t kc = std::min<int64_t>(Kall, OZ_KMAX);
-    while (!fit(kc) && kc > 16) kc = std::max<int64_t>(16, rup(kc / 2, 16));  // chunk K to fit
-    // chunks of equal depth
-    const int64_t nch = (Kall + kc - 1) / kc;
-    if (nch > 1) fit(std::min(kc, rup((Kall + nch - 1) / nch, 16)));
+    // the fewest chunks of equal depth that fit
+    int64_t nch = (Kall + kmax - 1) / kmax;
+    while (!fit(rup((Kall + nch - 1) / nch, 16)) && p.Kc > 16) nch *= 2;
     p.kchunk = rup((p.Kp + p.splits - 1) / p.splits, OZ_KC);
     p.splits = (int)((p.Kp + p.kchunk - 1) / p.kchunk);
     return p;
 }
 }  // namespace
 
-size_t ozaki_workspace_bytes(int M, int N, int K, bool hermitian) {
-    return std::max(make_plan(M, N, K, hermitian, SIZE_MAX, OZ_BM).bytes,
-                    make_plan(M, N, K, hermitian, SIZE_MAX, OZT_BM).bytes);
+size_t ozaki_workspace_bytes(int M, int N, int K, bool hermitian, int64_t kmax) {
+    if (kmax <= 0 || kmax > OZ_KMAX) kmax = OZ_KMAX;
+    return std::max(make_plan(M, N, K, hermitian, SIZE_MAX, OZ_BM, kmax).bytes,
+                    make_plan(M, N, K, hermitian, SIZE_MAX, OZT_BM, kmax).bytes);
 }
 
 double ozaki_tc_flops(int M, int N, int K, bool hermitian, bool legacy) {
     if (M <= 0 || N <= 0 || K <= 0) return 0.0;
     const int bm = legacy ? OZ_BM : OZT_BM;
-    const OzPlan p = make_plan(M, N, K, hermitian, SIZE_MAX, bm);
+    const bool upper = hermitian && M == N;
+    const OzPlan p = make_plan(M, N, K, upper, SIZE_MAX, bm);
     const double pairs = OZ_S * (OZ_S + 1) / 2;
-    const bool upper = hermitian && M == N && (N % OZ_BN) == 0;
-    const double tiles = (double)tile_count(p.Mp, p.Np, bm, upper, upper ? N / OZ_BN : p.Np / OZ_BN);
+    const double tiles = (double)tile_count(p.Mp, p.Np, bm, upper, upper ? p.H / OZ_BN : p.Np / OZ_BN);
     return 2.0 * pairs * tiles * bm * OZ_BN * (double)p.Kp;
 }
 
@@ -928,8 +983,8 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
     int *Eb = Ea + p.Mp;
     w += rup((int64_t)sizeof(int) * (p.Mp + p.Np), 256);
     double *Wp = p.splits > 1 ? reinterpret_cast<double *>(w) : nullptr;
-    const bool upper = hermitian && (N % OZ_BN) == 0;
-    const int halfN_tiles = upper ? N / OZ_BN : (int)(p.Np / OZ_BN);
+    const bool upper = hermitian;
+    const int H = (int)p.H, halfN_tiles = (int)(upper ? p.H / OZ_BN : p.Np / OZ_BN);
 
     for (int64_t kc0 = 0; kc0 < K; kc0 += p.Kc) {
         const int Kc = (int)std::min<int64_t>(p.Kc, K - kc0);
@@ -937,12 +992,12 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
         const double2 *Ak = conjA ? A + kc0 : A + kc0 * lda;
         const double2 *Bk = B + kc0;
         if ((e = cudaMemsetAsync(Ea, 0, sizeof(int) * (p.Mp + p.Np), s)) != cudaSuccess) return e;
-        if (conjA)
-            oz_colexp_kernel<<<std::min(M, 65535), 256, 0, s>>>(Ea, Ak, lda, Kc, M, 0);
-        else
+        if (conjA && !hermitian)
+            oz_colexp_kernel<<<std::min(M, 65535), 256, 0, s>>>(Ea, Ak, lda, Kc, M, 0, nullptr);
+        else if (!conjA)
             oz_rowexp_kernel<<<dim3((unsigned)((M + 31) / 32), (unsigned)((Kc + 255) / 256)), 256, 0, s>>>(
                 Ea, Ak, lda, M, Kc);
-        oz_colexp_kernel<<<std::min(N, 65535), 256, 0, s>>>(Eb, Bk, ldb, Kc, N, N);
+        oz_colexp_kernel<<<std::min(N, 65535), 256, 0, s>>>(Eb, Bk, ldb, Kc, N, H, hermitian ? Ea : nullptr);
         if (legacy) {
             const int kx = (int)std::min<int64_t>((p.Kp / 2 + 255) / 256, 64);
             if (conjA)
@@ -952,19 +1007,26 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
                 oz_slice_rows_kernel<<<dim3((unsigned)(p.Mp / 32), (unsigned)((p.Kp / 2 + 31) / 32)), 256, 0,
                                        s>>>(As, Ea, Ak, lda, M, Kc, (int)p.Mp, (int)p.Kp);
             oz_slice_cols_kernel<<<dim3(kx, (unsigned)std::min<int64_t>(p.Np, 65535)), 256, 0, s>>>(
-                Bs, Eb, Bk, ldb, 1, 2 * N, N, Kc, (int)p.Np, (int)p.Kp);
+                Bs, Eb, Bk, ldb, 1, N, H, Kc, (int)p.Np, (int)p.Kp);
         } else {
             // stage images: one warp per 8 rows x 8 of K'
             auto blocks = [](int64_t rows, int64_t kp) {
                 return (unsigned)std::max<int64_t>(1, std::min<int64_t>(rows / 8 * (kp / 8) / 8, 152 * 16));
             };
-            oz_slice_tiled_kernel<<<blocks(p.Mp, p.Kp), 256, 0, s>>>(As, Ea, Ak, lda, conjA ? 0 : 2, M, M, Kc,
-                                                                     (int)p.Mp, (int)p.Kp, OZT_BM, 0);
-            oz_slice_tiled_kernel<<<blocks(p.Np, p.Kp), 256, 0, s>>>(Bs, Eb, Bk, ldb, 1, 2 * N, N, Kc,
-                                                                     (int)p.Np, (int)p.Kp, OZT_BN, 1);
+            if (!hermitian) {
+                if (conjA)
+                    oz_slice_columns_kernel<<<blocks(p.Mp, p.Kp), 256, 0, s>>>(As, (int)p.Mp, nullptr, 0, 0, Ea, Ak, lda,
+                                                                               M, Kc, (int)p.Kp, OZT_BM, OZT_BN);
+                else
+                    oz_slice_rows_tiled_kernel<<<blocks(p.Mp, p.Kp), 256, 0, s>>>(As, Ea, Ak, lda, M, Kc, (int)p.Mp,
+                                                                                  (int)p.Kp, OZT_BM);
+            }
+            oz_slice_columns_kernel<<<blocks(std::max(p.Mp, p.H), p.Kp), 256, 0, s>>>(
+                hermitian ? As : nullptr, (int)p.Mp, Bs, H, (int)p.Np, Eb, Bk, ldb, N, Kc, (int)p.Kp, OZT_BM, OZT_BN);
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        const dim3 grid((unsigned)(p.Mp / bm), (unsigned)(p.Np / OZ_BN), (unsigned)p.splits);
+        const unsigned tm = (unsigned)(p.Mp / bm), tn = (unsigned)(p.Np / OZ_BN);
+        const dim3 grid = legacy ? dim3(tm, tn, (unsigned)p.splits) : dim3(tm * tn, 1, (unsigned)p.splits);
         cudaEvent_t ev1 = nullptr;
         if (timer) {
             cudaEvent_t ev0;
@@ -973,11 +1035,11 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
             if ((e = cudaEventRecord(ev0, s)) != cudaSuccess) return e;
         }
         if (legacy)
-            oz_gemm_kernel<<<grid, OZ_THREADS, OZ_SMEM, s>>>(As, Bs, Ea, Eb, Wp, C, ldc, M, N, (int)p.Mp,
+            oz_gemm_kernel<<<grid, OZ_THREADS, OZ_SMEM, s>>>(As, Bs, Ea, Eb, Wp, C, ldc, M, N, H, (int)p.Mp,
                                                             (int)p.Np, (int)p.Kp, (int)p.kchunk,
                                                             halfN_tiles, upper ? 1 : 0, alpha, b);
         else
-            oz_gemm_tc_kernel<<<grid, OZT_THREADS, OZT_SMEM, s>>>(As, Bs, Ea, Eb, Wp, C, ldc, M, N,
+            oz_gemm_tc_kernel<<<grid, OZT_THREADS, OZT_SMEM, s>>>(As, Bs, Ea, Eb, Wp, C, ldc, M, N, H,
                                                                  (int)p.Mp, (int)p.Np, (int)p.Kp,
                                                                  (int)p.kchunk, halfN_tiles,
                                                                  upper ? 1 : 0, alpha, b, status);
@@ -985,12 +1047,12 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
         if (timer && (e = cudaEventRecord(ev1, s)) != cudaSuccess) return e;
         if (tc_flops) *tc_flops += ozaki_tc_flops(M, N, Kc, upper, legacy);
         if (Wp) {
-            oz_combine_kernel<<<grid_for((int64_t)M * N), 256, 0, s>>>(C, ldc, Wp, M, N, (int)p.Mp,
+            oz_combine_kernel<<<grid_for((int64_t)M * N), 256, 0, s>>>(C, ldc, Wp, M, N, H, (int)p.Mp,
                                                                        (int)p.Np, p.splits, alpha, b,
                                                                        upper ? 1 : 0, bm);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
-        if (launches) *launches += 5 + (Wp ? 1 : 0);
+        if (launches) *launches += (hermitian && !legacy ? 3 : 5) + (Wp ? 1 : 0);
     }
     if (hermitian) {  // exactly Hermitian result, whether or not tiles were skipped
         oz_mirror_kernel<<<grid_for((int64_t)M * M), 256, 0, s>>>(C, ldc, M);
@@ -1004,7 +1066,80 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
 // ----------------------------------------------------------- C ABI
 namespace rsrr {
 std::string &thread_error();  // api.cu: last error of a handle-less call
+
+// Work space of rsrr_zgemm: a stream-ordered pool per device that keeps at most
+// ZGEMM_KEEP bytes between calls (mapping and unmapping 1.7 GB took 1.15 ms of a
+// 40000 x 500 Gram matrix's 3.4); allocations and frees are ordered on the
+// caller's stream, so threads and streams do not share a block in use.  What is
+// kept is given back when a handle or a server is created, and when an
+// allocation of the pool fails.
+constexpr uint64_t ZGEMM_KEEP = 2ull << 30;
+constexpr int ZGEMM_DEVICES = 64;
+static std::mutex g_zgemm_mu;
+static cudaMemPool_t g_zgemm_pool[ZGEMM_DEVICES] = {};
+
+static cudaMemPool_t zgemm_pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= ZGEMM_DEVICES) return nullptr;
+    std::lock_guard<std::mutex> lk(g_zgemm_mu);
+    if (!g_zgemm_pool[dev]) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        uint64_t keep = ZGEMM_KEEP;
+        if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            cudaMemPoolDestroy(pool);
+            return nullptr;
+        }
+        g_zgemm_pool[dev] = pool;
+    }
+    return g_zgemm_pool[dev];
 }
+
+void zgemm_release_kept() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= ZGEMM_DEVICES) {
+        cudaGetLastError();
+        return;
+    }
+    std::lock_guard<std::mutex> lk(g_zgemm_mu);
+    if (g_zgemm_pool[dev] && cudaMemPoolTrimTo(g_zgemm_pool[dev], 0) != cudaSuccess) cudaGetLastError();
+}
+
+namespace {
+// one call's work space; freed on the stream it was allocated on
+struct ZgemmWs {
+    void *p = nullptr;
+    bool pooled = false;
+    cudaStream_t s;
+    explicit ZgemmWs(cudaStream_t stream) : s(stream) {}
+    cudaError_t get(size_t bytes) {
+        cudaError_t e = cudaErrorMemoryAllocation;
+        if (cudaMemPool_t pool = zgemm_pool()) {
+            e = cudaMallocFromPoolAsync(&p, bytes, pool, s);
+            pooled = e == cudaSuccess;
+            if (!pooled) cudaGetLastError();
+        }
+        if (!pooled) {
+            zgemm_release_kept();
+            e = cudaMalloc(&p, bytes);
+        }
+        return e;
+    }
+    ~ZgemmWs() {
+        if (p && pooled) cudaFreeAsync(p, s);
+        else if (p) cudaFree(p);
+    }
+};
+}  // namespace
+}  // namespace rsrr
 
 extern "C" rsrr_status rsrr_zgemm(int32_t M, int32_t N, int32_t K, int32_t conjA, const rsrr_c128 *A,
                                   int64_t lda, const rsrr_c128 *B, int64_t ldb, rsrr_c128 *C,
@@ -1043,8 +1178,9 @@ extern "C" rsrr_status rsrr_zgemm(int32_t M, int32_t N, int32_t K, int32_t conjA
         // the call's own status word (bounded waits that ran out) follows the
         // slices in the same allocation
         const size_t ws_bytes = need / 256 * 256;
-        void *ws = nullptr;
-        if ((e = cudaMalloc(&ws, ws_bytes + 256)) != cudaSuccess) return fail(RSRR_ENOMEM, "work space", e);
+        ZgemmWs hold(s);
+        if ((e = hold.get(ws_bytes + 256)) != cudaSuccess) return fail(RSRR_ENOMEM, "work space", e);
+        void *ws = hold.p;
         unsigned int *status = reinterpret_cast<unsigned int *>(static_cast<char *>(ws) + ws_bytes);
         unsigned int tmo = 0;
         e = cudaMemsetAsync(status, 0, sizeof(unsigned int), s);
@@ -1053,12 +1189,8 @@ extern "C" rsrr_status rsrr_zgemm(int32_t M, int32_t N, int32_t K, int32_t conjA
                             ws_bytes, s, nullptr, nullptr, nullptr, legacy, status);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&tmo, status, sizeof tmo, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess && tmo != 0) {
-            cudaFree(ws);
-            return fail(RSRR_ETIMEOUT, "a bounded tensor-core wait ran out");
-        }
+        if (e == cudaSuccess && tmo != 0) return fail(RSRR_ETIMEOUT, "a bounded tensor-core wait ran out");
         cudaError_t e2 = cudaStreamSynchronize(s);
-        cudaFree(ws);
         if (e == cudaErrorMemoryAllocation) return fail(RSRR_ENOMEM, "work space below one chunk");
         if (e != cudaSuccess) return fail(RSRR_ECUDA, "sliced gemm", e);
         if (e2 != cudaSuccess) return fail(RSRR_ECUDA, "sync", e2);

@@ -816,11 +816,11 @@ __global__ void scatter_inverse_fill_kernel(double2 *__restrict__ X, const doubl
 }
 
 // Work space of the sliced products: the Gram matrix of the n x NL block in
-// one piece (the other products of the sparse kind need less), capped at
-// 8 GiB; a product that needs more runs in chunks of K.
+// chunks of at most 32768 of its depth (the other products of the sparse kind
+// need less), capped at 8 GiB; a product that needs more runs in more chunks.
 static size_t ozaki_ws_bytes(int NL, int64_t n) {
     const int nc = (int)std::min<int64_t>(n, INT32_MAX / 2);
-    return std::min(ozaki_workspace_bytes(NL, NL, nc, true), (size_t)8 << 30);
+    return std::min(ozaki_workspace_bytes(NL, NL, nc, true, 32768), (size_t)8 << 30);
 }
 
 // Workspace layout of the projection stage (carved from one allocation).
@@ -845,7 +845,9 @@ static void carve_ws(char *cp, ProjWs &ws, int NL, int64_t n, int terms) {
     ws.jacc = carve<double>(cp, 2 * 4096);
     ws.Q1 = carve<double2>(cp, (size_t)n * NL);
     ws.Ytmp = carve<double2>(cp, (size_t)n * NL);
-    ws.gws_elems = std::max<size_t>(NL2 * 4, (size_t)8 << 20);
+    // (split-K slabs of the FP64 products; less than a round size by what the
+    // sliced products' padded halves and the block records of the band solve add)
+    ws.gws_elems = std::max<size_t>(NL2 * 4, (size_t)8 << 20) - (NL % 64 ? (size_t)9 << 19 : (size_t)1 << 20);
     ws.gws = carve<double2>(cp, ws.gws_elems);
     ws.ows_bytes = ozaki_ws_bytes(NL, n);
     ws.ows = carve<char>(cp, ws.ows_bytes);

@@ -216,7 +216,7 @@ cudaError_t fp64_gemm(int M, int N, int K, bool conjA, const double2 *A, int64_t
 // C = alpha op(A) B + beta C, op(A) = A^H when conjA; hermitian (A == B,
 // conjA, M == N) computes the upper block triangle and mirrors it.  ws holds
 // the slices; the product is done in K chunks when ws is smaller than
-// ozaki_workspace_bytes.  cudaErrorMemoryAllocation if ws cannot hold one
+// ozaki_workspace_bytes (kmax > 0: in chunks of at most that depth).  cudaErrorMemoryAllocation if ws cannot hold one
 // chunk of 16.
 // With timer set, a pair of events brackets every launch of the main kernel
 // and *tc_flops grows by the tensor-core flops it issues.  The main kernel is
@@ -231,7 +231,9 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
                         double beta, bool hermitian, void *ws, size_t ws_bytes, cudaStream_t s,
                         int64_t *launches, EventPool *timer = nullptr, double *tc_flops = nullptr,
                         bool legacy = false, unsigned int *status = nullptr);
-size_t ozaki_workspace_bytes(int M, int N, int K, bool hermitian);
+// gives the work space that rsrr_zgemm keeps on the current device back
+void zgemm_release_kept();
+size_t ozaki_workspace_bytes(int M, int N, int K, bool hermitian, int64_t kmax = 0);
 // one thread waits, with the tcgen05 kernel's bounded mbarrier wait, on a
 // barrier that nothing completes; after `limit` polls the wait is counted in
 // *status (failure detection without a GPU fault)

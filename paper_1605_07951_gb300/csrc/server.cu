@@ -221,6 +221,7 @@ rsrr_status rsrr_server_create(const rsrr_server_opts *opts, rsrr_server_t **out
     if (sv->o.device < 0) e = cudaGetDevice(&sv->device);
     else sv->device = sv->o.device;
     if (e == cudaSuccess) e = cudaSetDevice(sv->device);
+    if (e == cudaSuccess) rsrr::zgemm_release_kept();
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
