@@ -26,10 +26,13 @@ namespace rsrr {
 // op(A) = A (M x K) or A^H (A is K x M).  64x64 tiles, 256 threads with 4x4
 // outputs each, K slabs of 16 through shared memory, optional split-K into a
 // workspace (deterministic reduction) and optional upper-tile-only mode for
-// Hermitian products (the lower triangle is mirrored afterwards).
+// Hermitian products (the lower triangle is mirrored afterwards).  Few columns
+// take 64 x 16 tiles: the kernel is bound by the FP64 unit, where the lanes of a
+// padded column cost as much as the others.
 // ==========================================================================
 constexpr int GT = 64, GK = 16;
 
+template <int GN>
 __global__ void __launch_bounds__(256)
 zgemm_kernel(int M, int N, int K, bool conjA, const double2 *__restrict__ A, int64_t lda,
              const double2 *__restrict__ B, int64_t ldb, double2 *__restrict__ Cout, int64_t ldc,
@@ -37,16 +40,17 @@ zgemm_kernel(int M, int N, int K, bool conjA, const double2 *__restrict__ A, int
     const int bm = blockIdx.x, bn = blockIdx.y, ks = blockIdx.z;
     if (upper_only && bm > bn) return;
     __shared__ double2 As[GK][GT + 1];
-    __shared__ double2 Bs[GK][GT + 1];
+    constexpr int CB = GN / 16;  // columns of a thread
+    __shared__ double2 Bs[GK][GN + 1];
     const int tid = threadIdx.x;
     const int tx = tid % 16, ty = tid / 16;  // outputs rows tx+16a, cols ty+16b
-    const int m0 = bm * GT, n0 = bn * GT;
+    const int m0 = bm * GT, n0 = bn * GN;
     const int kbeg = ks * kchunk, kend = min(K, kbeg + kchunk);
-    double2 acc[4][4];
+    double2 acc[4][CB];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = make_double2(0.0, 0.0);
+        for (int b = 0; b < CB; ++b) acc[a][b] = make_double2(0.0, 0.0);
     for (int k0 = kbeg; k0 < kend; k0 += GK) {
         // A tile: op(A)(m0+i, k0+kk)
         for (int q = tid; q < GT * GK; q += 256) {
@@ -64,7 +68,7 @@ zgemm_kernel(int M, int N, int K, bool conjA, const double2 *__restrict__ A, int
             }
             As[kk][i] = v;
         }
-        for (int q = tid; q < GT * GK; q += 256) {
+        for (int q = tid; q < GN * GK; q += 256) {
             const int kk = q % GK, j = q / GK;
             double2 v = make_double2(0.0, 0.0);
             if (n0 + j < N && k0 + kk < kend) v = B[(int64_t)(n0 + j) * ldb + (k0 + kk)];
@@ -73,15 +77,15 @@ zgemm_kernel(int M, int N, int K, bool conjA, const double2 *__restrict__ A, int
         __syncthreads();
 #pragma unroll 4
         for (int kk = 0; kk < GK; ++kk) {
-            double2 av[4], bv[4];
+            double2 av[4], bv[CB];
 #pragma unroll
             for (int a = 0; a < 4; ++a) av[a] = As[kk][tx + 16 * a];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][ty + 16 * b];
+            for (int b = 0; b < CB; ++b) bv[b] = Bs[kk][ty + 16 * b];
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = cfma(acc[a][b], av[a], bv[b]);
+                for (int b = 0; b < CB; ++b) acc[a][b] = cfma(acc[a][b], av[a], bv[b]);
         }
         __syncthreads();
     }
@@ -89,7 +93,7 @@ zgemm_kernel(int M, int N, int K, bool conjA, const double2 *__restrict__ A, int
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
+        for (int b = 0; b < CB; ++b) {
             const int i = m0 + tx + 16 * a, j = n0 + ty + 16 * b;
             if (i < M && j < N) {
                 double2 r = make_double2(alpha * acc[a][b].x, alpha * acc[a][b].y);
@@ -139,7 +143,7 @@ static int grid1d(int64_t work, int threads = 256) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 8));
 }
 
-// workspace-backed GEMM: chooses split-K so that enough CTAs run
+// workspace-backed GEMM: chooses split-K so that whole waves of SMs run
 struct Gemm {
     double2 *ws = nullptr;
     size_t ws_elems = 0;
@@ -174,16 +178,25 @@ struct Gemm {
             if (e == cudaSuccess && timer) e = cudaEventRecord(ev1, s);
             return e;
         }
-        const int tm = (M + GT - 1) / GT, tn = (N + GT - 1) / GT;
-        int64_t tiles = hermitian ? (int64_t)tm * (tm + 1) / 2 : (int64_t)tm * tn;
+        const bool narrow = N <= 48 && !hermitian;
+        const int gn = narrow ? 16 : GT;
+        const int tm = (M + GT - 1) / GT, tn = (N + gn - 1) / gn;
+        const int64_t tiles = hermitian ? (int64_t)tm * (tm + 1) / 2 : (int64_t)tm * tn;
+        // splits of K that fill whole waves of SMs (the FP64 unit of an SM is
+        // shared by its CTAs, so a wave costs its depth).  Below the line of the
+        // sliced products, the 16 products of an SS-RR solve of order 3600: 12.0
+        // -> 6.6 ms, where two CTAs an SM and at most K / 256 splits stood before
+        // and every tile had 64 columns
         int splits = 1;
-        const int64_t target = 152 * 2;
-        if (tiles < target && K > 4 * GK) {
-            splits = (int)std::min<int64_t>((target + tiles - 1) / tiles, (K + 255) / 256);
-            while (splits > 1 && (size_t)splits * M * N > ws_elems) --splits;
+        double best = 1e300;
+        for (int q = 1; q <= 64 && q * 64 <= std::max(K, 64); ++q) {
+            if (q > 1 && (size_t)q * M * N > ws_elems) break;
+            const double cost = (double)((tiles * q + 151) / 152) / q * (1.0 + 0.01 * q);
+            if (cost < best - 1e-12) {
+                best = cost;
+                splits = q;
+            }
         }
-        if (K <= 0) splits = 1;
-        if (splits > 1 && (size_t)splits * M * N > ws_elems) splits = 1;
         int kchunk = (K + splits - 1) / splits;
         kchunk = ((kchunk + GK - 1) / GK) * GK;
         if (kchunk < GK) kchunk = GK;
@@ -200,11 +213,11 @@ struct Gemm {
         }
         if (counter) *counter += 1 + (splits == 1 ? 0 : 1) + (hermitian ? 1 : 0);
         if (splits == 1) {  // direct: the kernel writes C itself
-            zgemm_kernel<<<grid, 256, 0, s>>>(M, N, K, conjA, A, lda, B, ldb, C, ldc, kchunk,
-                                              hermitian, alpha, beta);
+            (narrow ? zgemm_kernel<16> : zgemm_kernel<GT>)<<<grid, 256, 0, s>>>(M, N, K, conjA, A, lda, B, ldb, C, ldc,
+                                                                               kchunk, hermitian, alpha, beta);
         } else {
-            zgemm_kernel<<<grid, 256, 0, s>>>(M, N, K, conjA, A, lda, B, ldb, ws, M, kchunk,
-                                              hermitian, 1.0, 0.0);
+            (narrow ? zgemm_kernel<16> : zgemm_kernel<GT>)<<<grid, 256, 0, s>>>(M, N, K, conjA, A, lda, B, ldb, ws, M,
+                                                                               kchunk, hermitian, 1.0, 0.0);
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;
             splitk_reduce_kernel<<<grid1d((int64_t)M * N), 256, 0, s>>>(
