@@ -299,34 +299,28 @@ __global__ void diag_real_kernel(double *__restrict__ d, const double2 *__restri
 
 // ==========================================================================
 // Bounded grid-wide barrier for cooperative launches (all CTAs co-resident).
-// bar[0] arrivals, bar[1] generation, bar[2] error flag.  A CTA that waits
-// more than 2^24 polls (~2 s) sets the error flag; every CTA then stops.
-// Returns false once the flag is set.
+// bar[0] arrivals since the launch (zeroed before it; never reset within, so an
+// arrival is one atomic and a waiter polls the counter itself), bar[2] error
+// flag.  A CTA that waits more than 2^22 polls (~2 s) sets the error flag and
+// stops; the others find it while they wait for that CTA.  Returns false then.
 // ==========================================================================
-constexpr long long GRID_WAIT_LIMIT = 1LL << 24;
+constexpr int GRID_WAIT_LIMIT = 1 << 22;
 
 RSRR_DEV bool grid_sync(unsigned int *bar, unsigned int nblocks) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned int *vb = bar;
-        const unsigned int gen = vb[1];
-        __threadfence();
+        unsigned int v;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(bar) : "memory");
+        const unsigned int want = (v / nblocks + 1) * nblocks;
         int ok = 1;
-        if (atomicAdd(bar, 1u) == nblocks - 1) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-        } else {
-            long long it = 0;
-            while (vb[1] == gen) {
-                if (vb[2]) { ok = 0; break; }
-                if (++it > GRID_WAIT_LIMIT) { atomicExch(bar + 2, 1u); ok = 0; break; }
-                __nanosleep(64);
-            }
+        ++v;
+        for (int it = 0; (int)(v - want) < 0; ++it) {
+            if ((it & 15) == 15 && *(volatile unsigned int *)(bar + 2)) { ok = 0; break; }
+            if (it >= GRID_WAIT_LIMIT) { atomicExch(bar + 2, 1u); ok = 0; break; }
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
         }
-        __threadfence();
-        s_ok = ok && !vb[2];
+        s_ok = ok;
     }
     __syncthreads();
     return s_ok != 0;
@@ -370,7 +364,8 @@ RSRR_DEV void block_argmax(const double *__restrict__ d, int n, double &bv, int 
 // Column j costs n j complex FMAs on the FP64 unit: a block takes 32 rows, its
 // eight warps an eighth of the earlier columns each (a row per thread kept n /
 // 256 SMs busy), partial sums added in warp order.  The four factorisations of an
-// SS-RR solve of order 40000 with 2048 moment columns: 12.5 -> 4.1 ms.
+// SS-RR solve of order 40000 with 2048 moment columns: 12.5 -> 4.1 ms, 3.5 ms with
+// the barrier of one atomic.
 __global__ void __launch_bounds__(256)
 pchol_persistent_kernel(const double2 *__restrict__ G, int n, double2 *__restrict__ Lm,
                         double *__restrict__ dbuf, double tau, int32_t *__restrict__ state,
@@ -433,26 +428,29 @@ pchol_persistent_kernel(const double2 *__restrict__ G, int n, double2 *__restric
 // sweep).  Each thread owns a 2x2 block (pair a, pair b) of H and rewrites it
 // as J_a^H H J_b, reading the old matrix and writing the new one (double
 // buffer); the rotations come from the old matrix.  Y <- Y J in place.
-// Rotation for [[alpha, beta], [conj(beta), gamma]], beta = |beta| e^{i phi}:
-//   tau = (gamma - alpha) / (2|beta|), t = sign(tau)/(|tau| + sqrt(1+tau^2)),
-//   c = 1/sqrt(1+t^2), s = t c,  J = [[c, s e^{i phi}], [-s e^{-i phi}, c]].
+// Rotation for [[alpha, beta], [conj(beta), gamma]], d = (gamma - alpha) / 2,
+// w = |d| + sqrt(d^2 + |beta|^2), r = 1 / sqrt(w^2 + |beta|^2):
+//   J = [[c, se], [-conj(se), c]],  c = w r,  se = sign(d) beta r.
 // ==========================================================================
 struct Rot {
     double c;
-    double2 se;  // s e^{i phi}
+    double2 se;
 };
 
 RSRR_DEV void pair_of(int r, int a, int kp, int &p, int &q) {
     if (a == 0) {
         p = kp - 1;
         q = r;
-    } else {
-        p = (r + a) % (kp - 1);
-        q = (r - a + (kp - 1)) % (kp - 1);
+    } else {  // 0 <= r < kp - 1, 1 <= a < kp - 1
+        p = r + a - (r + a >= kp - 1 ? kp - 1 : 0);
+        q = r - a + (r < a ? kp - 1 : 0);
     }
     if (p > q) { const int t = p; p = q; q = t; }
 }
 
+// One square root and one reciprocal square root: an instruction of the FP64 unit
+// costs a warp 64 cycles, and every CTA waits for its round's rotations.  d and
+// beta are scaled by a power of two so that their squares stay in range.
 RSRR_DEV Rot rot_of(const double2 *__restrict__ H, int k, int p, int q) {
     Rot R;
     R.c = 1.0;
@@ -460,24 +458,33 @@ RSRR_DEV Rot rot_of(const double2 *__restrict__ H, int k, int p, int q) {
     if (p >= k || q >= k) return R;
     const double al = H[(int64_t)p * k + p].x, ga = H[(int64_t)q * k + q].x;
     const double2 be = H[(int64_t)q * k + p];  // H(p, q)
-    const double ab = hypot(be.x, be.y);
-    if (ab <= 1e-300 || ab <= 1e-18 * sqrt(fabs(al * ga))) return R;
-    const double tau = (ga - al) / (2.0 * ab);
-    const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-    const double c = 1.0 / sqrt(1.0 + t * t), s = t * c;
-    R.c = c;
-    R.se = make_double2(s * be.x / ab, s * be.y / ab);
+    const double d = 0.5 * (ga - al);
+    const int eb = max(__double2hiint(be.x) & 0x7fffffff, __double2hiint(be.y) & 0x7fffffff) >> 20;
+    const int ed = max(eb, (__double2hiint(d) & 0x7fffffff) >> 20);
+    if (eb < 27) return R;  // |beta| below 2^-996
+    const int sc = min(max(2046 - ed, 1), 2046);  // 2^(1023 - ed), exponent field
+    const double f = __hiloint2double(sc << 20, 0);
+    const double ds = d * f, bx = be.x * f, by = be.y * f;
+    const double b2 = fma(bx, bx, by * by);
+    if (b2 <= 1e-36 * fabs((al * f) * (ga * f))) return R;
+    const double w = fabs(ds) + sqrt(fma(ds, ds, b2));
+    const double ri = rsqrt(fma(w, w, b2)), sg = ds >= 0.0 ? ri : -ri;
+    R.c = w * ri;
+    R.se = make_double2(sg * bx, sg * by);
     return R;
 }
 
-// One round of the round-robin ordering, grid-stride over the 2x2 blocks and
-// the rows of Y.  Every CTA first computes the round's np rotations (one per
-// pair, from the old matrix) into shared memory `srot`, so that the FP64
-// square roots and divisions run once per pair rather than once per block.
+// One round of the round-robin ordering, grid-stride over the elements of the
+// 2x2 blocks and the rows of Y.  Every CTA first computes the round's np rotations
+// (one per pair, from the old matrix) into shared memory `srot`.  Only the blocks
+// a <= b are computed, the others are their conjugates; an element of a block to
+// a thread, since the FP64 unit charges for a warp's instructions and not for its
+// lanes.  The two decompositions of an SS-RR solve of order 3600: 9.7 -> 4.8 ms, of
+// order 40000: 17.0 -> 8.8 ms (with the barrier of one atomic above).
 RSRR_DEV void jacobi_round(const double2 *__restrict__ Hold, double2 *__restrict__ Hnew,
                            double2 *__restrict__ Y, int k, int kp, int r, Rot *__restrict__ srot) {
     const int np = kp / 2;
-    const int64_t nblk = (int64_t)np * np;
+    const int64_t nH = (int64_t)np * (np + 1) * 2;  // 4 elements x np (np + 1) / 2 blocks
     const int64_t nY = (int64_t)k * np;
     for (int a = threadIdx.x; a < np; a += blockDim.x) {
         int p, q;
@@ -485,54 +492,48 @@ RSRR_DEV void jacobi_round(const double2 *__restrict__ Hold, double2 *__restrict
         srot[a] = rot_of(Hold, k, p, q);
     }
     __syncthreads();
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nblk + nY;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        if (q < nblk) {
-            const int a = (int)(q % np), b = (int)(q / np);
+    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nH + nY;
+         g += (int64_t)gridDim.x * blockDim.x) {
+        if (g < nH) {
+            const int e = (int)g & 1, f = ((int)g >> 1) & 1;  // element (e, f) of the block
+            const unsigned int blk = (unsigned int)(g >> 2), wd = np | 1;
+            const int R = (int)(blk / wd), c = (int)(blk % wd);
+            // rows np-1-R and R (np even) or R-1 (np odd) of the triangle share a row of wd blocks
+            const bool first = c < np - R;
+            const int b = first ? np - 1 - R : R - (np & 1), a = first ? c : c - (np - R);
             int pa, qa, pb, qb;
             pair_of(r, a, kp, pa, qa);
             pair_of(r, b, kp, pb, qb);
             const Rot Ra = srot[a], Rb = srot[b];
-            const bool va = qa < k, vb = qb < k;
-            double2 h00 = (pa < k && pb < k) ? Hold[(int64_t)pb * k + pa] : make_double2(0, 0);
-            double2 h01 = (pa < k && vb) ? Hold[(int64_t)qb * k + pa] : make_double2(0, 0);
-            double2 h10 = (va && pb < k) ? Hold[(int64_t)pb * k + qa] : make_double2(0, 0);
-            double2 h11 = (va && vb) ? Hold[(int64_t)qb * k + qa] : make_double2(0, 0);
-            const double cb = Rb.c;
-            const double2 sb = Rb.se, sbc = make_double2(-sb.x, sb.y);
-            double2 t00 = cadd(make_double2(h00.x * cb, h00.y * cb), cmul(h01, sbc));
-            double2 t01 = cadd(cmul(h00, sb), make_double2(h01.x * cb, h01.y * cb));
-            double2 t10 = cadd(make_double2(h10.x * cb, h10.y * cb), cmul(h11, sbc));
-            double2 t11 = cadd(cmul(h10, sb), make_double2(h11.x * cb, h11.y * cb));
-            const double ca = Ra.c;
-            const double2 sa = Ra.se, msa = make_double2(-sa.x, -sa.y), sac = make_double2(sa.x, -sa.y);
-            double2 n00 = cadd(make_double2(t00.x * ca, t00.y * ca), cmul(msa, t10));
-            double2 n01 = cadd(make_double2(t01.x * ca, t01.y * ca), cmul(msa, t11));
-            double2 n10 = cadd(cmul(sac, t00), make_double2(t10.x * ca, t10.y * ca));
-            double2 n11 = cadd(cmul(sac, t01), make_double2(t11.x * ca, t11.y * ca));
+            const int row = e ? qa : pa, rowo = e ? pa : qa, col = f ? qb : pb, colo = f ? pb : qb;
+            if (row >= k || col >= k) continue;
+            const double2 zero = make_double2(0.0, 0.0);
+            const double2 h_ss = Hold[(int64_t)col * k + row];
+            const double2 h_so = colo < k ? Hold[(int64_t)colo * k + row] : zero;
+            const double2 h_os = rowo < k ? Hold[(int64_t)col * k + rowo] : zero;
+            const double2 h_oo = (rowo < k && colo < k) ? Hold[(int64_t)colo * k + rowo] : zero;
+            // column col of H J: c_b h(., col) + z h(., colo); row `row` of J^H (H J) alike
+            const double2 z = f ? Rb.se : make_double2(-Rb.se.x, Rb.se.y);
+            const double2 w = e ? make_double2(Ra.se.x, -Ra.se.y) : make_double2(-Ra.se.x, -Ra.se.y);
+            const double2 ts = cfma(make_double2(h_ss.x * Rb.c, h_ss.y * Rb.c), h_so, z);
+            const double2 to = cfma(make_double2(h_os.x * Rb.c, h_os.y * Rb.c), h_oo, z);
+            double2 n = cfma(make_double2(ts.x * Ra.c, ts.y * Ra.c), to, w);
             if (a == b) {
-                n00.y = 0.0;
-                n11.y = 0.0;
-                if (Ra.se.x != 0.0 || Ra.se.y != 0.0) {
-                    n01 = make_double2(0.0, 0.0);
-                    n10 = make_double2(0.0, 0.0);
-                }
+                if (e == f) n.y = 0.0;
+                else if (Ra.se.x != 0.0 || Ra.se.y != 0.0) n = zero;
             }
-            if (pa < k && pb < k) Hnew[(int64_t)pb * k + pa] = n00;
-            if (pa < k && vb) Hnew[(int64_t)qb * k + pa] = n01;
-            if (va && pb < k) Hnew[(int64_t)pb * k + qa] = n10;
-            if (va && vb) Hnew[(int64_t)qb * k + qa] = n11;
+            Hnew[(int64_t)col * k + row] = n;
+            if (a != b) Hnew[(int64_t)row * k + col] = make_double2(n.x, -n.y);
         } else {
-            const int64_t w = q - nblk;
-            const int i = (int)(w % k), b = (int)(w / k);
+            const unsigned int w = (unsigned int)(g - nH);
+            const int i = (int)(w % (unsigned int)k), b = (int)(w / (unsigned int)k);
             int pb, qb;
             pair_of(r, b, kp, pb, qb);
             if (qb >= k) continue;
             const Rot Rb = srot[b];
             const double2 yp = Y[(int64_t)pb * k + i], yq = Y[(int64_t)qb * k + i];
-            const double2 sbc = make_double2(-Rb.se.x, Rb.se.y);
-            Y[(int64_t)pb * k + i] = cadd(make_double2(yp.x * Rb.c, yp.y * Rb.c), cmul(yq, sbc));
-            Y[(int64_t)qb * k + i] = cadd(cmul(yp, Rb.se), make_double2(yq.x * Rb.c, yq.y * Rb.c));
+            Y[(int64_t)pb * k + i] = cfma(make_double2(yp.x * Rb.c, yp.y * Rb.c), yq, make_double2(-Rb.se.x, Rb.se.y));
+            Y[(int64_t)qb * k + i] = cfma(make_double2(yq.x * Rb.c, yq.y * Rb.c), yp, Rb.se);
         }
     }
 }
@@ -540,7 +541,7 @@ RSRR_DEV void jacobi_round(const double2 *__restrict__ Hold, double2 *__restrict
 // Whole cyclic Jacobi in one cooperative launch: Y = I, then sweeps of
 // kp-1 rounds (grid barrier after each), convergence test after each sweep
 // (off(H)^2 <= tol2 * diag(H)^2 from per-CTA partial sums in acc, one slot
-// pair per CTA, added in CTA order).  The final matrix is copied back into
+// pair per CTA, added in one order).  The final matrix is copied back into
 // H0.  state[0] = sweeps run.
 __global__ void __launch_bounds__(256)
 jacobi_persistent_kernel(double2 *__restrict__ H0, double2 *__restrict__ H1,
@@ -572,26 +573,32 @@ jacobi_persistent_kernel(double2 *__restrict__ H0, double2 *__restrict__ H1,
                 if ((q % k) == (q / k)) dia += m2; else off += m2;
             }
             // deterministic reduction: per-CTA partials in fixed slots, summed
-            // in CTA order by every CTA after the barrier
+            // in one order by every CTA after the barrier
             __shared__ double s_off[8], s_dia[8];
-            for (int o = 16; o; o >>= 1) {
-                off += shfl_down(off, o);
-                dia += shfl_down(dia, o);
-            }
-            if ((threadIdx.x & 31) == 0) { s_off[threadIdx.x >> 5] = off; s_dia[threadIdx.x >> 5] = dia; }
-            __syncthreads();
+            auto block_sums = [&](double x, double y, double &sx, double &sy) {
+                for (int o = 16; o; o >>= 1) {
+                    x += shfl_down(x, o);
+                    y += shfl_down(y, o);
+                }
+                __syncthreads();
+                if ((threadIdx.x & 31) == 0) { s_off[threadIdx.x >> 5] = x; s_dia[threadIdx.x >> 5] = y; }
+                __syncthreads();
+                sx = sy = 0.0;
+                for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { sx += s_off[w]; sy += s_dia[w]; }
+            };
+            double o2, d2;
+            block_sums(off, dia, o2, d2);
             if (threadIdx.x == 0) {
-                double a = 0.0, b2 = 0.0;
-                for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { a += s_off[w]; b2 += s_dia[w]; }
-                acc[2 * blockIdx.x] = a;
-                acc[2 * blockIdx.x + 1] = b2;
+                acc[2 * blockIdx.x] = o2;
+                acc[2 * blockIdx.x + 1] = d2;
             }
             if (!grid_sync(bar, gridDim.x)) return;
-            double o2 = 0.0, d2 = 0.0;
-            for (int c = 0; c < (int)gridDim.x; ++c) {
-                o2 += *((volatile double *)(acc + 2 * c));
-                d2 += *((volatile double *)(acc + 2 * c + 1));
+            off = dia = 0.0;
+            for (int c = threadIdx.x; c < (int)gridDim.x; c += blockDim.x) {
+                off += *((volatile double *)(acc + 2 * c));
+                dia += *((volatile double *)(acc + 2 * c + 1));
             }
+            block_sums(off, dia, o2, d2);
             const bool done = o2 <= tol2 * d2;
             if (!grid_sync(bar, gridDim.x)) return;  // acc is rewritten next sweep
             if (done) break;
@@ -728,13 +735,13 @@ static cudaError_t jacobi_eig(ProjWs &ws, int k, cudaStream_t s, int64_t *counte
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.jacc, 0, sizeof(double) * 2 * 4096, s);
     if (e != cudaSuccess) return e;
     const double tol2 = 1e-30;  // off(H) <= 1e-15 ||diag(H)||
-    const int64_t work = (int64_t)(k + 1) / 2 * ((k + 1) / 2) + (int64_t)k * ((k + 1) / 2);
+    const int64_t np = (k + 1) / 2, work = 2 * np * (np + 1) + k * np;
     const size_t smem = sizeof(Rot) * (size_t)((k + 1) / 2);
     // at most one CTA per SM: the round's work is FP64-bound per SM either way,
     // and fewer arrivals make the grid barrier after every round cheaper
     int dev = 0, nsm = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    e = launch_coop_smem(jacobi_persistent_kernel, (int)std::min<int64_t>((work + 255) / 256, nsm), smem,
+    e = launch_coop_smem(jacobi_persistent_kernel, (int)std::min<int64_t>((work + 127) / 128, nsm), smem,
                          s, ws.H, ws.H2, ws.Y, k, max_sweeps, tol2, ws.jacc, ws.state + 1, ws.bar);
     if (e != cudaSuccess) return e;
     sort_desc_kernel<<<1, 256, 0, s>>>(ws.H, k, ws.order, ws.evals);
