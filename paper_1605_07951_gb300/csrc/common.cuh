@@ -140,6 +140,9 @@ RSRR_DEV float crecip(float b) { return 1.f / b; }
 RSRR_DEV double crecip(double b) { return 1.0 / b; }
 
 template <typename T> RSRR_DEV T shfl_down(T v, int off) { return __shfl_down_sync(0xffffffffu, v, off); }
+template <typename T> RSRR_DEV T cshfl(T v, int src) {  // a complex value from lane src
+    return T{__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src)};
+}
 
 // max of non-negative doubles through their ordered bit patterns
 RSRR_DEV void atomic_max_nonneg(double *addr, double v) {

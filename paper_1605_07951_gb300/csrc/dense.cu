@@ -10,6 +10,7 @@
 // never to the columns already factored: the solve applies each block's
 // interchanges just before that block's elimination, as the band solve does.
 #include <algorithm>
+#include <climits>
 #include <type_traits>
 
 #include "common.cuh"
@@ -163,7 +164,273 @@ __global__ void dense_tnorm_kernel(double *__restrict__ tnorm, const double2 *__
 constexpr int DP_THREADS = 1024;
 constexpr int DP_WARPS = DP_THREADS / 32;
 
-// Panel k0 (columns k0..k0+jb-1, rows k0..n-1) of every point, one CTA per
+// Inverses of the unit lower L11 and of U11 of the diagonal block at k0 (jb x jb,
+// zero padded to NB x NB), for the solve.  A lane per row: a warp carries 32 / NB
+// columns of an inverse, each step broadcasts one entry of it by shuffle and
+// updates the rows below (above).  rinv: the reciprocals of the diagonal of U11.
+template <typename C, int NB, int WARPS>
+RSRR_DEV void panel_inverses(const C *__restrict__ A, C *__restrict__ dst, C *__restrict__ s_blk,
+                             const C *__restrict__ rinv, int n, int k0, int jb) {
+    constexpr int CPW = 32 / NB, TASKS = NB / CPW;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int q = tid; q < NB * NB; q += 32 * WARPS) {
+        const int j = q / NB, i = q % NB;
+        s_blk[q] = (i < jb && j < jb) ? A[(int64_t)(k0 + j) * n + k0 + i] : czero<C>();
+    }
+    __syncthreads();
+    const int t = lane % NB, sub = lane / NB;
+    for (int task = warp; task < 2 * TASKS; task += WARPS) {
+        const bool lower = task < TASKS;
+        const int jf = (lower ? task : task - TASKS) * CPW, j = jf + sub;
+        C x = (t == j && j < jb) ? cone<C>() : czero<C>();
+        if (lower) {
+            for (int i = jf; i < jb - 1; ++i) {
+                const C xi = cshfl(x, (lane & ~(NB - 1)) + i);
+                if (i >= j && t > i) x = cfms(x, s_blk[i * NB + t], xi);
+            }
+        } else {
+            for (int i = min(jf + CPW, jb) - 1; i >= 0; --i) {
+                const C xi = cmul(cshfl(x, (lane & ~(NB - 1)) + i), rinv[i]);
+                if (i <= j && t == i) x = xi;
+                if (i <= j && t < i) x = cfms(x, s_blk[i * NB + t], xi);
+            }
+        }
+        dst[(lower ? 0 : NB * NB) + j * NB + t] = (t < jb && j < jb) ? x : czero<C>();
+    }
+}
+
+// |re|+|im| as an ordered integer (never NaN), and the largest of a warp with the
+// first row that has it: redux on integers, where compares of doubles would each
+// cost the warp 64 cycles of the FP64 unit
+RSRR_DEV int panel_key(float v) {
+    const int b = __float_as_int(v) & 0x7fffffff;
+    return b > 0x7f800000 ? 0 : b;
+}
+RSRR_DEV long long panel_key(double v) {
+    const long long b = __double_as_longlong(v) & 0x7fffffffffffffffll;
+    return b > 0x7ff0000000000000ll ? 0 : b;
+}
+RSRR_DEV int panel_best(int &key, int row) {
+    const int m = __reduce_max_sync(0xffffffffu, key);
+    row = __reduce_min_sync(0xffffffffu, key == m ? row : INT_MAX);
+    key = m;
+    return row;
+}
+RSRR_DEV int panel_best(long long &key, int row) {
+    const int hi = (int)(key >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned lo = hi == mh ? (unsigned)key : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+    row = __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? row : INT_MAX);
+    key = ((long long)mh << 32) | ml;
+    return row;
+}
+
+// Panel k0 (columns k0..k0+jb-1, rows k0..n-1, at most T * RPT of them) of every
+// point, one CTA per point.  Bound by the chain of its columns, so the rows live in
+// registers (RPT a thread), W columns at a time, and a column costs one barrier:
+// before it every warp publishes the row of its largest |re|+|im| (first row on
+// ties) and the owner of the pivot's place its row, after it every thread finds the
+// winner, exchanges, and updates its rows with the winner's.  Where W < NB, the
+// panel's other columns take the W interchanges, the triangular solve and the
+// rank-W update from global memory afterwards.  In complex128 one warp takes the
+// reciprocal (its three divisions by every warp cost as much as the update) behind
+// a second barrier.  The operations on an element and their order are those of
+// dense_panel_kernel below.  All panels of a factorisation, against that kernel:
+// complex64, 32 points of order 500 2.3 -> 0.68 ms, of order 2048 16.0 -> 5.3 ms;
+// complex128, 512 nodes of order 237 15.8 -> 1.5 ms.
+template <typename C, int NB, int W, int RPT, int T>
+__global__ void __launch_bounds__(T, 512 / T)
+dense_panel_reg_kernel(C *__restrict__ A_all, int32_t *__restrict__ piv_all, int32_t *__restrict__ info_all,
+                       C *__restrict__ dinv_all, int n, int k0) {
+    using R = typename real_of<C>::type;
+    using Key = decltype(panel_key(R()));
+    constexpr int NW = T / 32, GW = W < 8 ? W : 8;
+    static_assert(2 * W * (NB - W) <= T, "one element of the interchanged rows per thread");
+    constexpr bool FP64 = sizeof(R) == 8;
+    const int pt = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    C *A = A_all + (size_t)pt * n * n + (size_t)k0 * n;  // column k0
+    int32_t *piv = piv_all + (size_t)pt * n;
+    const int jb = min(NB, n - k0);
+    __shared__ Key s_key[2][NW];
+    __shared__ int s_idx[2][NW], s_p[W];
+    __shared__ C s_cand[2][NW][W], s_own[2][W], s_piv[W][W], s_u[W][NB], s_rinv[NB], s_blk[NB * NB];
+    int par = 0;
+    for (int s0 = 0; s0 < jb; s0 += W) {
+        const int wj = min(W, jb - s0);
+        C a[RPT][W];
+        Key key = -1;
+        int row = INT_MAX;
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            const int r = k0 + tid + q * T;
+#pragma unroll
+            for (int j = 0; j < W; ++j)
+                a[q][j] = (r < n && r >= k0 + s0 && j < wj) ? A[(int64_t)(s0 + j) * n + r] : czero<C>();
+        }
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            const int r = k0 + tid + q * T;
+            if (r < n && r >= k0 + s0) {
+                const Key k = panel_key(cabs1(a[q][0]));
+                if (k > key) { key = k; row = r; }
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < W / GW; ++g) {
+#pragma unroll 1
+            for (int u = 0; u < GW; ++u) {
+                const int cc = g * GW + u, c = k0 + s0 + cc;
+                if (cc >= wj) break;
+                Key wk = key;
+                const int wr = panel_best(wk, row);
+                if (lane == 0) { s_key[par][warp] = wk; s_idx[par][warp] = wr; }
+#pragma unroll
+                for (int q = 0; q < RPT; ++q) {
+                    const int r = k0 + tid + q * T;
+                    if (r == wr)
+#pragma unroll
+                        for (int j = 0; j < W; ++j) s_cand[par][warp][j] = a[q][j];
+                    if (r == c)
+#pragma unroll
+                        for (int j = 0; j < W; ++j) s_own[par][j] = a[q][j];
+                }
+                __syncthreads();
+                Key bk = lane < NW ? s_key[par][lane] : -1;
+                const int p = panel_best(bk, lane < NW ? s_idx[par][lane] : INT_MAX);
+                const C *pr = s_cand[par][((p - k0) % T) >> 5];
+                const C pv = pr[cc];
+                C inv;
+                if constexpr (FP64) {
+                    if (warp == 0) {
+                        inv = crecip(pv);
+                        if (lane == 0) s_rinv[s0 + cc] = inv;
+                    }
+                } else {
+                    inv = crecip(pv);
+                    if (tid == 0) s_rinv[s0 + cc] = inv;
+                }
+                if (tid < W) s_piv[cc][tid] = pr[tid];
+                if (tid == 0) {
+                    s_p[cc] = p;
+                    piv[c] = p;
+                    if (bk <= 0 && info_all[pt] == 0) info_all[pt] = c + 1;
+                }
+                if constexpr (FP64) {
+                    __syncthreads();
+                    inv = s_rinv[s0 + cc];
+                }
+                key = -1;
+                row = INT_MAX;
+                const bool nz = cnonzero(pv);
+#pragma unroll
+                for (int q = 0; q < RPT; ++q) {
+                    const int r = k0 + tid + q * T;
+                    if (r == p && p != c)
+#pragma unroll
+                        for (int j = 0; j < W; ++j) a[q][j] = s_own[par][j];
+                    if (r > c && r < n) {
+                        if (nz) {
+                            C l = a[q][g * GW];
+#pragma unroll
+                            for (int v = 1; v < GW; ++v)
+                                if (v == u) l = a[q][g * GW + v];
+                            l = cmul(l, inv);
+#pragma unroll
+                            for (int v = 0; v < GW; ++v)
+                                if (v == u) a[q][g * GW + v] = l;
+#pragma unroll
+                            for (int j = g * GW + 1; j < W; ++j)
+                                if (j > cc) a[q][j] = cfms(a[q][j], l, pr[j]);
+                        }
+                        C nx = czero<C>();
+#pragma unroll
+                        for (int v = g * GW + 1; v < W && v <= g * GW + GW; ++v)
+                            if (v == cc + 1) nx = a[q][v];
+                        const Key k = panel_key(cabs1(nx));
+                        if (k > key) { key = k; row = r; }
+                    }
+                }
+                par ^= 1;
+            }
+        }
+        const int top = k0 + s0 + wj;
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            const int r = k0 + tid + q * T;
+            if (r >= top && r < n)
+#pragma unroll
+                for (int j = 0; j < W; ++j)
+                    if (j < wj) A[(int64_t)(s0 + j) * n + r] = a[q][j];
+        }
+        __syncthreads();
+        for (int e = tid; e < wj * wj; e += T) {
+            const int i = e % wj, j = e / wj;
+            A[(int64_t)(s0 + j) * n + k0 + s0 + i] = s_piv[i][j];
+        }
+        if constexpr (W < NB) {
+            // interchanges of the other columns: the row that ends at x started at y
+            C val = czero<C>();
+            const int col = tid / (2 * wj), slot = tid % (2 * wj);
+            const int oc = col < s0 ? col : col + wj;  // column of the panel
+            int x = 0;
+            const bool mine = col < jb - wj;
+            if (mine) {
+                x = slot < wj ? k0 + s0 + slot : s_p[slot - wj];
+                int y = x;
+                for (int i = wj - 1; i >= 0; --i) {
+                    const int ci = k0 + s0 + i, pi = s_p[i];
+                    y = y == ci ? pi : (y == pi ? ci : y);
+                }
+                val = A[(int64_t)oc * n + y];
+            }
+            __syncthreads();
+            if (mine) {
+                A[(int64_t)oc * n + x] = val;
+                if (slot < wj) s_u[slot][oc] = val;
+            }
+            __syncthreads();
+            const int rest = jb - s0 - wj;  // columns to the right; wj == W if there are any
+            if (tid < rest) {
+                const int oc2 = s0 + wj + tid;
+                C uu[W];
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    uu[i] = s_u[i][oc2];
+#pragma unroll
+                    for (int t = 0; t < i; ++t) uu[i] = cfms(uu[i], s_piv[i][t], uu[t]);
+                    s_u[i][oc2] = uu[i];
+                    A[(int64_t)oc2 * n + k0 + s0 + i] = uu[i];
+                }
+            }
+            __syncthreads();
+#pragma unroll 2
+            for (int c2 = s0 + wj; c2 < jb; ++c2) {
+                C xv[RPT];
+#pragma unroll
+                for (int q = 0; q < RPT; ++q) {
+                    const int r = k0 + tid + q * T;
+                    xv[q] = (r >= top && r < n) ? A[(int64_t)c2 * n + r] : czero<C>();
+                }
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    const C ui = s_u[i][c2];
+#pragma unroll
+                    for (int q = 0; q < RPT; ++q) xv[q] = cfms(xv[q], a[q][i], ui);
+                }
+#pragma unroll
+                for (int q = 0; q < RPT; ++q) {
+                    const int r = k0 + tid + q * T;
+                    if (r >= top && r < n) A[(int64_t)c2 * n + r] = xv[q];
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const size_t nblk = ((size_t)n + NB - 1) / NB;
+    panel_inverses<C, NB, NW>(A - (size_t)k0 * n, dinv_all + ((size_t)pt * nblk + k0 / NB) * 2 * NB * NB, s_blk, s_rinv,
+                              n, k0, jb);
+}
+
+// Panels of more rows than the registers of an SM hold: one CTA per
 // point, right-looking in global memory (L2): per column a block-wide argmax
 // of |re|+|im| (first index on ties), the interchange inside the panel, the
 // multipliers and the rank-1 update of the remaining panel columns.  Then
@@ -182,7 +449,7 @@ dense_panel_kernel(C *__restrict__ A_all, int32_t *__restrict__ piv_all, int32_t
     __shared__ int s_i[DP_WARPS];
     __shared__ C s_row[NB];
     __shared__ C s_blk[NB * NB];
-    __shared__ C s_inv[2][NB * (NB + 1)];
+    __shared__ C s_rinv[NB];
     for (int cc = 0; cc < jb; ++cc) {
         const int c = k0 + cc;
         R v = (R)-1;
@@ -202,6 +469,7 @@ dense_panel_kernel(C *__restrict__ A_all, int32_t *__restrict__ piv_all, int32_t
         int p = s_i[0];
         for (int w = 1; w < DP_WARPS; ++w)
             if (s_v[w] > bv || (s_v[w] == bv && s_i[w] < p)) { bv = s_v[w]; p = s_i[w]; }
+        if (p >= n) p = c;  // a column of NaN
         if (tid < jb && p != c) {
             const int64_t col = (int64_t)(k0 + tid) * n;
             const C t = A[col + c]; A[col + c] = A[col + p]; A[col + p] = t;
@@ -227,38 +495,23 @@ dense_panel_kernel(C *__restrict__ A_all, int32_t *__restrict__ piv_all, int32_t
         }
         __syncthreads();
     }
-    // diagonal block inverses
-    for (int q = tid; q < NB * NB; q += DP_THREADS) {
-        const int j = q / NB, i = q % NB;
-        s_blk[q] = (i < jb && j < jb) ? A[(int64_t)(k0 + j) * n + k0 + i] : czero<C>();
-    }
-    __syncthreads();
-    if (warp == 0 && lane < NB) {
-        const int j = lane;  // column j of L11^{-1}
-        for (int i = 0; i < NB; ++i) {
-            C s = (i == j) ? cone<C>() : czero<C>();
-            for (int t = j; t < i; ++t) s = cfms(s, s_blk[t * NB + i], s_inv[0][j * (NB + 1) + t]);
-            s_inv[0][j * (NB + 1) + i] = (i < j || i >= jb || j >= jb) ? czero<C>() : s;
-        }
-    } else if (warp == 1 && lane < NB) {
-        const int j = lane;  // column j of U11^{-1}
-        for (int i = 0; i < NB; ++i) s_inv[1][j * (NB + 1) + i] = czero<C>();
-        if (j < jb) {
-            s_inv[1][j * (NB + 1) + j] = crecip(s_blk[j * NB + j]);
-            for (int i = j - 1; i >= 0; --i) {
-                C s = czero<C>();
-                for (int t = i + 1; t <= j; ++t) s = cfma(s, s_blk[t * NB + i], s_inv[1][j * (NB + 1) + t]);
-                s_inv[1][j * (NB + 1) + i] = cmul(csub(czero<C>(), s), crecip(s_blk[i * NB + i]));
-            }
-        }
-    }
-    __syncthreads();
-    const int nblk = (n + NB - 1) / NB;
-    C *dst = dinv_all + ((size_t)pt * nblk + k0 / NB) * 2 * NB * NB;
-    for (int q = tid; q < 2 * NB * NB; q += DP_THREADS) {
-        const int w = q / (NB * NB), e = q % (NB * NB), j = e / NB, i = e % NB;
-        dst[q] = s_inv[w][j * (NB + 1) + i];
-    }
+    if (tid < jb) s_rinv[tid] = crecip(A[(int64_t)(k0 + tid) * n + k0 + tid]);
+    const size_t nblk = ((size_t)n + NB - 1) / NB;
+    panel_inverses<C, NB, DP_WARPS>(A, dinv_all + ((size_t)pt * nblk + k0 / NB) * 2 * NB * NB, s_blk, s_rinv, n, k0, jb);
+}
+
+// Rows in registers while they fit (64 registers a thread, up to 4096 rows), 256
+// threads where they suffice, so that two panels share an SM.
+template <typename C, int NB>
+static void dense_panel(C *A, int32_t *piv, int32_t *info, C *dinv, int n, int k0, int N, cudaStream_t s) {
+    constexpr int W1 = 256 / (int)sizeof(C) < NB ? 256 / (int)sizeof(C) : NB;
+    const int rows = n - k0;
+    if (rows <= 256) dense_panel_reg_kernel<C, NB, W1, 1, 256><<<N, 256, 0, s>>>(A, piv, info, dinv, n, k0);
+    else if (rows <= 512) dense_panel_reg_kernel<C, NB, W1, 1, 512><<<N, 512, 0, s>>>(A, piv, info, dinv, n, k0);
+    else if (rows <= 1024) dense_panel_reg_kernel<C, NB, W1 / 2, 2, 512><<<N, 512, 0, s>>>(A, piv, info, dinv, n, k0);
+    else if (rows <= 2048) dense_panel_reg_kernel<C, NB, W1 / 4, 4, 512><<<N, 512, 0, s>>>(A, piv, info, dinv, n, k0);
+    else if (rows <= 4096) dense_panel_reg_kernel<C, NB, W1 / 8, 8, 512><<<N, 512, 0, s>>>(A, piv, info, dinv, n, k0);
+    else dense_panel_kernel<C, NB><<<N, DP_THREADS, 0, s>>>(A, piv, info, dinv, n, k0);
 }
 
 // Trailing columns k0+jb.. in chunks of 32: the panel's interchanges (in
@@ -785,7 +1038,7 @@ static cudaError_t dense_lu_t(C *A, int32_t *piv, int32_t *info, C *dinv, int n,
     if (e != cudaSuccess) return e;
     for (int k0 = 0; k0 < n; k0 += NB) {
         const int jb = std::min(NB, n - k0);
-        dense_panel_kernel<C, NB><<<N, DP_THREADS, 0, s>>>(A, piv, info, dinv, n, k0);
+        dense_panel<C, NB>(A, piv, info, dinv, n, k0, N, s);
         const int rest = n - k0 - jb;
         if (rest > 0) {
             dense_laswp_trsm_kernel<C, NB><<<dim3((rest + 31) / 32, N), 256, 0, s>>>(A, piv, dinv, n, k0);
