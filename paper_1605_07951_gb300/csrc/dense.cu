@@ -20,59 +20,61 @@ namespace rsrr {
 
 constexpr double kFourPi = 12.566370614359172;
 
-RSRR_DEV void store_d(float2 *p, double2 v) { *p = to_c64(v); }
-RSRR_DEV void store_d(double2 *p, double2 v) { *p = v; }
-
 // ---------------------------------------------------------------- assembly
-// complex64 entries from FP32 sincos/exp (the factor is complex64 anyway);
-// complex128 entries in FP64 (used by the FP64 residual and the FP64 path).
-__global__ void assemble_dense_c64_kernel(float2 *__restrict__ A_all, const double *__restrict__ pts,
-                                          const double2 *__restrict__ zs, double diag, int n) {
-    const int pt = blockIdx.y;
-    const float zr = (float)zs[pt].x, zi = (float)zs[pt].y;
-    float2 *A = A_all + (size_t)pt * n * n;
-    const int64_t total = (int64_t)n * n;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(q / n), i = (int)(q - (int64_t)j * n);
-        float2 v;
-        if (i == j) {
-            v = make_float2((float)diag, 0.f);
-        } else {
-            const float dx = (float)(pts[3 * i] - pts[3 * j]), dy = (float)(pts[3 * i + 1] - pts[3 * j + 1]),
-                        dz = (float)(pts[3 * i + 2] - pts[3 * j + 2]);
-            const float r = sqrtf(dx * dx + dy * dy + dz * dz);
-            const float mag = expf(-zi * r) / ((float)kFourPi * r);
-            float s, c;
-            sincosf(zr * r, &s, &c);
-            v = make_float2(mag * c, mag * s);
-        }
-        A[q] = v;
-    }
-}
+// FP64 entries; the mixed path's complex64 matrix is narrowed from them.  T is
+// symmetric (r_ij and r_ji have the same bits), so a block takes a pair of 32 x 32
+// tiles: the entries with j >= i are computed, kept in shared memory and written to
+// both.  Bound by the FP64 unit (exp, sincos and a division per entry): a lane per
+// entry, the distances once for all points of the block, the transcendentals half as
+// often as there are entries.  32 points of order 2048: 16.4 -> 6.7 ms.
+constexpr int AT = 32;
 
-__global__ void assemble_dense_c128_kernel(double2 *__restrict__ A_all, const double *__restrict__ pts,
-                                           const double2 *__restrict__ zs, double diag, int n) {
-    const int pt = blockIdx.y;
-    const double zr = zs[pt].x, zi = zs[pt].y;
-    double2 *A = A_all + (size_t)pt * n * n;
-    const int64_t total = (int64_t)n * n;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(q / n), i = (int)(q - (int64_t)j * n);
-        double2 v;
-        if (i == j) {
-            v = make_double2(diag, 0.0);
-        } else {
+__global__ void __launch_bounds__(256)
+assemble_dense_kernel(double2 *__restrict__ A_all, const double *__restrict__ pts, const double2 *__restrict__ zs,
+                      double diag, int n, int N) {
+    __shared__ double2 s_t[AT][AT + 1];
+    // tile pair (bi <= bj) of the upper triangle
+    int bj = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+    while ((int64_t)(bj + 1) * (bj + 2) / 2 <= blockIdx.x) ++bj;
+    while ((int64_t)bj * (bj + 1) / 2 > blockIdx.x) --bj;
+    const int bi = (int)(blockIdx.x - (int64_t)bj * (bj + 1) / 2);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = bi * AT + lane;
+    double r[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int j = bj * AT + warp + 8 * q;
+        r[q] = -1.0;
+        if (i < n && j < n && i < j) {
             const double dx = pts[3 * i] - pts[3 * j], dy = pts[3 * i + 1] - pts[3 * j + 1],
                          dz = pts[3 * i + 2] - pts[3 * j + 2];
-            const double r = sqrt(dx * dx + dy * dy + dz * dz);
-            const double mag = exp(-zi * r) / (kFourPi * r);
-            double s, c;
-            sincos(zr * r, &s, &c);
-            v = make_double2(mag * c, mag * s);
+            r[q] = sqrt(dx * dx + dy * dy + dz * dz);
         }
-        A[q] = v;
+    }
+    for (int pt = blockIdx.y; pt < N; pt += gridDim.y) {
+        const double zr = zs[pt].x, zi = zs[pt].y;
+        double2 *A = A_all + (size_t)pt * n * n;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int jj = warp + 8 * q, j = bj * AT + jj;
+            if (i >= n || j >= n || i > j) continue;
+            double2 v = make_double2(diag, 0.0);
+            if (i < j) {
+                const double mag = exp(-zi * r[q]) / (kFourPi * r[q]);
+                double s, c;
+                sincos(zr * r[q], &s, &c);
+                v = make_double2(mag * c, mag * s);
+            }
+            s_t[jj][lane] = v;
+            A[(int64_t)j * n + i] = v;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {  // column i2 of the mirrored tile, rows j2
+            const int ii = warp + 8 * q, i2 = bi * AT + ii, j2 = bj * AT + lane;
+            if (j2 < n && i2 < j2) A[(int64_t)i2 * n + j2] = s_t[lane][ii];
+        }
     }
 }
 
@@ -148,16 +150,35 @@ __global__ void col_norms2_kernel(const double2 *__restrict__ R, const double2 *
     }
 }
 
-// ||T(z_j)||_inf from the stored complex128 matrix: row sums of moduli
-__global__ void dense_tnorm_kernel(double *__restrict__ tnorm, const double2 *__restrict__ A_all, int n) {
-    const int pt = blockIdx.y;
+// |v| without hypot's scaling where the squares stay in range
+RSRR_DEV double cabs_fast(double2 v) {
+    const int hx = __double2hiint(v.x) & 0x7fffffff, hy = __double2hiint(v.y) & 0x7fffffff, h = max(hx, hy);
+    if (h >= (600 << 20) && h < (1400 << 20)) return sqrt(fma(v.x, v.x, v.y * v.y));
+    if ((hx | hy | __double2loint(v.x) | __double2loint(v.y)) == 0) return 0.0;
+    return cabsv(v);
+}
+
+// ||T(z_j)||_inf from the stored complex128 matrix: row sums of moduli.  A block
+// takes 32 rows, its eight warps every eighth column each (a thread per row left the
+// SMs to 500 warps for 32 points of order 500): that order 0.59 -> 0.20 ms, order
+// 2048 4.8 -> 2.7 ms.
+__global__ void __launch_bounds__(256)
+dense_tnorm_kernel(double *__restrict__ tnorm, const double2 *__restrict__ A_all, int n) {
+    __shared__ double s_sum[8][32];
+    const int pt = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double2 *A = A_all + (size_t)pt * n * n;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * 32 + lane;
     double s = 0.0;
     if (i < n)
-        for (int j = 0; j < n; ++j) s += cabsv(A[(int64_t)j * n + i]);
-    for (int off = 16; off; off >>= 1) s = fmax(s, shfl_down(s, off));
-    if ((threadIdx.x & 31) == 0) atomic_max_nonneg(tnorm + pt, s);
+#pragma unroll 4
+        for (int j = warp; j < n; j += 8) s += cabs_fast(A[(int64_t)j * n + i]);
+    s_sum[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0) {
+        for (int w = 1; w < 8; ++w) s += s_sum[w][lane];
+        for (int off = 16; off; off >>= 1) s = fmax(s, shfl_down(s, off));
+        if (lane == 0) atomic_max_nonneg(tnorm + pt, s);
+    }
 }
 
 // ---------------------------------------------------------------- LU
@@ -973,16 +994,14 @@ static int grid_for_d(int64_t work, int threads = 256, int cap = 152 * 16) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, cap));
 }
 
-cudaError_t launch_assemble_dense_c64(float2 *A, const double *pts, const double2 *zs, double diag,
-                                      int n, int N, cudaStream_t s) {
-    assemble_dense_c64_kernel<<<dim3(grid_for_d((int64_t)n * n, 256, 2048), N), 256, 0, s>>>(A, pts, zs,
-                                                                                          diag, n);
-    return cudaGetLastError();
-}
 cudaError_t launch_assemble_dense_c128(double2 *A, const double *pts, const double2 *zs, double diag,
                                        int n, int N, cudaStream_t s) {
-    assemble_dense_c128_kernel<<<dim3(grid_for_d((int64_t)n * n, 256, 2048), N), 256, 0, s>>>(A, pts,
-                                                                                           zs, diag, n);
+    const int64_t nt = ((int64_t)n + AT - 1) / AT, pairs = nt * (nt + 1) / 2;
+    if (pairs > 0x7fffffff) return cudaErrorInvalidValue;
+    // blocks of one tile pair share its distances over their points: enough blocks for
+    // eight waves, more points each beyond that
+    const int64_t groups = std::max<int64_t>(1, std::min<int64_t>(std::min(N, 65535), 152 * 8 * 8 / pairs));
+    assemble_dense_kernel<<<dim3((unsigned)pairs, (unsigned)groups), 256, 0, s>>>(A, pts, zs, diag, n, N);
     return cudaGetLastError();
 }
 cudaError_t launch_assemble_dense_terms(double2 *T, const double2 *A, const double2 *coef, int n, int N,
@@ -1013,7 +1032,7 @@ cudaError_t launch_col_norms2(const double2 *R, const double2 *V, int n, int cnt
 cudaError_t launch_dense_tnorm(double *tnorm, const double2 *A, int n, int N, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(tnorm, 0, sizeof(double) * N, s);
     if (e != cudaSuccess) return e;
-    dense_tnorm_kernel<<<dim3((n + 255) / 256, N), 256, 0, s>>>(tnorm, A, n);
+    dense_tnorm_kernel<<<dim3((n + 31) / 32, N), 256, 0, s>>>(tnorm, A, n);
     return cudaGetLastError();
 }
 

@@ -125,8 +125,6 @@ cudaError_t launch_update(double2 *X, const float2 *D, int64_t per_pt, int N, co
                           cudaStream_t s);
 
 // ---- dense kernel path (dense.cu)
-cudaError_t launch_assemble_dense_c64(float2 *A, const double *pts, const double2 *zs, double diag,
-                                      int n, int N, cudaStream_t s);
 cudaError_t launch_assemble_dense_c128(double2 *A, const double *pts, const double2 *zs, double diag,
                                        int n, int N, cudaStream_t s);
 cudaError_t launch_dense_tnorm(double *tnorm, const double2 *A, int n, int N, cudaStream_t s);
