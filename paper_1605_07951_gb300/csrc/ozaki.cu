@@ -28,6 +28,7 @@
 //    K' <= 98304 keeps it below 2^62.6 (K is chunked beyond 49152).
 // 4. C~_ij = 2^(e_i + f_j) 2^-46 (acc + 2^32 low), rounded once to FP64.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdint>
 #include <cuda.h>
@@ -328,11 +329,19 @@ RSRR_DEV long long scaled_group_to_ll(float f) {
     return bits < 0 ? -m : m;
 }
 
-// 2^n (acc + 2^32 low), rounded once to FP64 in the sum.  The exponent is added
-// in integers: the FP64 unit, whose instructions take 64 cycles a warp, is left
-// with the two conversions and one FMA.
+// low (0 or at least 2^-48 in modulus) times 2^32 in FP64, by its bits
+RSRR_DEV double low_value(float low) {
+    const uint32_t b = (uint32_t)__float_as_int(low);
+    const uint32_t e = (b >> 23) & 0xFF;
+    if (e == 0 || e == 0xFF) return (double)low;  // zeros; infinities and NaN
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + ((896u + 32u) << 20))), (int)(b << 29));
+}
+
+// 2^n (acc + 2^32 low), rounded once to FP64 in the sum.  The exponent is added and
+// low converted in integers: the FP64 unit, whose instructions take 64 cycles a warp,
+// is left with one conversion and one addition.
 RSRR_DEV double oz_value(long long acc, float low, int n) {
-    const double d = fma((double)low, 0x1p32, (double)acc);
+    const double d = (double)acc + low_value(low);
     const long long b = __double_as_longlong(d);
     const int ex = (int)((b >> 52) & 0x7FF), nx = ex + n;
     if (ex >= 1 && ex <= 2046 && nx >= 1 && nx <= 2046) return __longlong_as_double(b + ((long long)n << 52));
@@ -480,44 +489,50 @@ oz_gemm_kernel(const __nv_bfloat16 *__restrict__ As, const __nv_bfloat16 *__rest
 }
 
 // ----------------------------------------------------------- tcgen05 path
-// The same products on the 5th-generation tensor cores: a CTA of 256 threads
-// owns a 128 x 64 tile of C~.  Per 16-deep stage of K' the 7 A slices (128
+// The same products on the 5th-generation tensor cores: one CTA an SM takes 128 x
+// 64 tiles of C~ in turn.  Per 16-deep stage of K' the 7 A slices (128
 // rows) and the 7 B slices (64 rows each, stacked to 448 rows) arrive by two
 // bulk copies of the TMA engine (the stage images of the slicing kernels,
 // 28 and 14 KB, contiguous in global memory; issued by one thread, completion
 // counted in bytes on the stage's mbarrier) in the K-major core-matrix layout
 // (8 rows x 16 bytes per core matrix, no swizzle), in a ring of OZT_NST
-// stages; a slot is refilled once the MMAs that read it have committed.  One thread issues
+// stages that runs on from tile to tile; a slot is refilled once the MMAs that read
+// it have committed.  One thread issues
 // 10 tcgen05.mma per stage (M = 128, N = 64..256, bf16 -> FP32 in tensor
 // memory): every group t = p + q has its own 64-column region of tensor
 // memory (7 regions, 448 of the 512 columns), so the pairs of one A slice
 // (q = 0 .. 6 - p) are MMAs over consecutive B slices into consecutive
-// regions, four slices (N = 256) at a time; the issuing thread never waits
-// at a CTA-wide barrier except for the folds.  Groups t <= 4 hold at most
-// (t+1) 2^14 per K' element, so every 192 of K' (and at the end) all threads
-// wait for the MMAs (tcgen05.commit -> mbarrier), read their part of the
+// regions, four slices (N = 256) at a time.  Groups t <= 4 hold at most
+// (t+1) 2^14 per K' element, so every 192 of K' (and at the end of a tile) sixteen
+// warps wait for the MMAs (tcgen05.commit -> mbarrier), read their part of the
 // regions (tcgen05.ld; warp w of 16 reads TMEM lanes 32 (w % 4) .. +31 = tile
 // rows, columns 16 (w / 4) .. +15), fold groups 0..4 into 64-bit integers and add
 // groups 5..6 (relative weight <= 2^-40, rounded by design) into an FP32 sum;
-// the next MMAs restart every region.  Every mbarrier wait is bounded; a wait that runs out is
-// counted in the caller's device status word, and from then on the CTA issues no further TMA copy
-// or MMA (the copy and MMA threads share an abort flag in shared memory; skipped stages still
-// commit their mbarriers so that the folds stay balanced), waits (bounded) for the copies it did
-// issue, and finishes without hanging.
+// the next MMAs restart every region.  The copy and MMA threads are warps of their
+// own, so while a tile's sums become FP64 results (12 000 cycles of the FP64 unit,
+// as long as the MMAs of a 15-stage tile) the next tile's first MMAs run.
+// Every mbarrier wait is bounded; a wait that runs out is
+// counted in the caller's device status word and raises an abort flag in shared memory, upon
+// which every role leaves its loop; the copies and MMAs already issued are waited for (bounded)
+// before the CTA ends.
+//
+// What it measured: with one tile a CTA, folds and results behind CTA-wide barriers, a
+// 30-stage tile took 100 000 cycles, 37 000 of them MMAs, 33 000 its results, 10 000
+// folds, the rest waits for the ring to fill: 40000 x 237 x 237 899 us, 500 x 500 x 40000
+// (Hermitian) 1534 us; now 534 and 1080 us.
 constexpr int OZT_BM = 128;
 constexpr int OZT_BN = 64;
 constexpr int OZT_KC = 16;
-constexpr int OZT_THREADS = 512;                 // 16 warps: 4 lane quarters x 4 column groups
-constexpr int OZT_CPT = OZT_BN / (OZT_THREADS / 128);  // tile columns a thread folds (16)
+constexpr int OZT_FOLDERS = 512;                 // 16 warps: 4 lane quarters x 4 column groups
+constexpr int OZT_THREADS = OZT_FOLDERS + 64;    // and a warp each for the MMAs and the copies
+constexpr int OZT_CPT = OZT_BN / (OZT_FOLDERS / 128);  // tile columns a thread folds (16)
 constexpr int OZT_GM = 8;                        // row tiles of a group (order of the tiles)
-constexpr int OZT_PRODUCER = OZT_THREADS / 2;    // the copy thread (first lane of the upper half)
 constexpr int OZT_A_SLICE = OZT_BM * OZT_KC * 2;           // bytes of one A slice per stage
 constexpr int OZT_B_SLICE = OZT_BN * OZT_KC * 2;           // bytes of one B slice per stage
 constexpr int OZT_STAGE = OZ_S * (OZT_A_SLICE + OZT_B_SLICE);
 constexpr int OZT_NST = 5;
-constexpr int OZT_DIST = OZT_NST - 2;  // stages the copies run ahead of a fold
-// after the stages: 2 NST + 1 mbarriers, the TMEM address, the abort flag
-constexpr int OZT_TSLOT = 16 * OZT_NST + 16;
+// after the stages: 2 NST + 3 mbarriers, the TMEM address, the abort flag
+constexpr int OZT_TSLOT = 16 * OZT_NST + 24;
 constexpr int OZT_ABORT = OZT_TSLOT + 16;
 constexpr size_t OZT_SMEM = (size_t)OZT_NST * OZT_STAGE + 128;
 static_assert(OZT_ABORT + 4 <= 128, "barrier area");
@@ -572,8 +587,8 @@ RSRR_DEV bool mbar_wait(uint32_t mbar, uint32_t parity, long long limit = OZT_WA
     return false;
 }
 // bounded wait that also gives up as soon as another thread of the CTA has
-// raised the abort flag (the copy and MMA threads; folds and the final drain
-// use the plain bounded wait so that operations in flight still land)
+// raised the abort flag, and raises it when it runs out (the final drain
+// uses the plain bounded wait so that operations in flight still land)
 RSRR_DEV bool mbar_wait_or_abort(uint32_t mbar, uint32_t parity, volatile int *abort_flag,
                                  long long limit = OZT_WAIT_LIMIT) {
     for (long long it = 0; it < limit; ++it) {
@@ -583,6 +598,7 @@ RSRR_DEV bool mbar_wait_or_abort(uint32_t mbar, uint32_t parity, volatile int *a
         if (done) return true;
         if (*abort_flag) return false;
     }
+    *abort_flag = 1;
     return false;
 }
 RSRR_DEV void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
@@ -610,37 +626,51 @@ RSRR_DEV int group_int(float g, float s12, float s) {
     return (int)(((uint32_t)__float_as_int(r) << 12) + (uint32_t)__float_as_int(r2) - 4097u * 0x4B400000u);
 }
 
+// the work list: split sp, row tile bm, column tile bn of item w of `tiles` per split.
+// Tiles go in groups of OZT_GM row tiles by all column tiles, row tiles first: the
+// CTAs at work together share few stage images of either operand, which
+// then come from L2.  Hermitian results: of each half the column tiles 2 bm ..
+RSRR_DEV void ozt_item(int w, int tiles, int nbm, int nbn, int halfN_tiles, int upper_only, int &sp, int &bm, int &bn) {
+    sp = w / tiles;
+    int t = w % tiles;
+    if (upper_only) {
+        bm = 0;
+        int cnt = halfN_tiles;  // column tiles of each half in row bm
+        while (t >= 2 * cnt) {
+            t -= 2 * cnt;
+            ++bm;
+            cnt -= OZT_BM / OZT_BN;
+        }
+        bn = (t / cnt) * halfN_tiles + (OZT_BM / OZT_BN) * bm + t % cnt;
+    } else {
+        const int grp = t / (OZT_GM * nbn), in = t % (OZT_GM * nbn);
+        const int gm = min(OZT_GM, nbm - grp * OZT_GM);  // the last group may be narrower
+        bm = grp * OZT_GM + in % gm;
+        bn = in / gm;
+    }
+}
+
 __global__ void __launch_bounds__(OZT_THREADS, 1)
 oz_gemm_tc_kernel(const __nv_bfloat16 *__restrict__ As, const __nv_bfloat16 *__restrict__ Bs,
                   const int *__restrict__ Ea, const int *__restrict__ Eb, double *__restrict__ W,
                   double2 *__restrict__ C, int64_t ldc, int M, int N, int H, int Mp, int Np, int Kp, int kchunk,
-                  int halfN_tiles, int upper_only, double alpha, double beta,
+                  int tiles, int items, int halfN_tiles, int upper_only, double alpha, double beta,
                   unsigned int *__restrict__ status) {
-    // tiles in groups of OZT_GM row tiles by all column tiles, row tiles first: the
-    // CTAs at work together share few stage images of either operand, which
-    // then come from L2 (column by column of tiles, a tall product read its
-    // A~ from DRAM once per column: 40000 x 237 x 237 909 -> 899 us)
-    const int nbm = Mp / OZT_BM, nbn = Np / OZT_BN;
-    const int grp = blockIdx.x / (OZT_GM * nbn), in = blockIdx.x % (OZT_GM * nbn);
-    const int gm = min(OZT_GM, nbm - grp * OZT_GM);  // the last group may be narrower
-    const int bm = grp * OZT_GM + in % gm, bn = in / gm, sp = blockIdx.z;
-    if (upper_only && OZT_BM * bm > OZT_BN * (bn % halfN_tiles) + OZT_BN - 1) return;
     extern __shared__ __align__(1024) unsigned char ozt_smem[];
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(ozt_smem);
     const uint32_t mb_full = sbase + OZT_NST * OZT_STAGE;  // OZT_NST: stage's bytes landed (TMA)
     const uint32_t mb_empty = mb_full + 8 * OZT_NST;       // OZT_NST: stage's MMAs done
     const uint32_t mb_fold = mb_empty + 8 * OZT_NST;       // all MMAs so far done
+    const uint32_t mb_free = mb_fold + 8;                  // regions read by the sixteen warps
+    const uint32_t mb_done = mb_free + 8;                  // the MMAs still in flight at the end
     uint32_t *tslot = reinterpret_cast<uint32_t *>(ozt_smem + OZT_NST * OZT_STAGE + OZT_TSLOT);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(ozt_smem + OZT_NST * OZT_STAGE + OZT_ABORT);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = bm * OZT_BM, n0 = bn * OZT_BN;
-    const int kbeg = sp * kchunk;
-    const int kend = min(Kp, kbeg + kchunk);
-    const int nk = kend > kbeg ? (kend - kbeg) / OZT_KC : 0;
-    // roles: thread OZT_PRODUCER copies the stages, thread 0 issues the MMAs,
-    // all sixteen warps fold (warp w: TMEM lanes 32 (w % 4) .., columns
-    // 16 (w / 4) ..)
-    const bool producer = tid >= OZT_PRODUCER;
+    const int nbm = Mp / OZT_BM, nbn = Np / OZT_BN;
+    auto stages = [&](int sp) {
+        const int kbeg = sp * kchunk, kend = min(Kp, kbeg + kchunk);
+        return kend > kbeg ? (kend - kbeg) / OZT_KC : 0;
+    };
 
     if (tid == 0) {
         for (int q = 0; q < OZT_NST; ++q) {
@@ -648,6 +678,8 @@ oz_gemm_tc_kernel(const __nv_bfloat16 *__restrict__ As, const __nv_bfloat16 *__r
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mb_empty + 8 * q));
         }
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mb_fold));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(mb_free), "n"(OZT_FOLDERS / 32));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mb_done));
         *abort_flag = 0;
     }
     if (warp == 0) {
@@ -659,137 +691,159 @@ oz_gemm_tc_kernel(const __nv_bfloat16 *__restrict__ As, const __nv_bfloat16 *__r
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = *tslot;
-    const int lrow = 32 * (warp & 3) + lane, lcol = OZT_CPT * (warp >> 2);
-    const uint32_t tpart = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)lcol;
-
-    long long acc[OZT_CPT];
-    float low[OZT_CPT];
-#pragma unroll
-    for (int c = 0; c < OZT_CPT; ++c) {
-        acc[c] = 0;
-        low[c] = 0.f;
-    }
     bool ok = true;
-    int folds = 0;
-    auto is_fold = [&](int st) { return ((st + 1) % OZT_FOLD) == 0 || st == nk - 1; };
-    // every warp, after the MMAs of a fold stage: regions 0..4 into the integers
-    auto fold_part = [&]() {
-        if (!mbar_wait(mb_fold, folds & 1)) {
-            ok = false;
-            *abort_flag = 1;
-        }
-        ++folds;
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        static_assert(OZT_CPT == 16, "one 16-column TMEM load per region");
+
+    if (warp == OZT_FOLDERS / 32) {  // ---- the MMAs
+        if (lane == 0) {
+            int slot = 0, folds = 0;
+            uint32_t phase = 0;
+            const uint64_t da = umma_desc(sbase, OZT_LBO_A), db = umma_desc(sbase + OZ_S * OZT_A_SLICE, OZT_LBO_B);
+            for (int w = blockIdx.x; ok && w < items; w += gridDim.x) {
+                int sp, bm, bn;
+                ozt_item(w, tiles, nbm, nbn, halfN_tiles, upper_only, sp, bm, bn);
+                const int nk = stages(sp);
+                for (int it = 0, left = 0; it < nk; ++it) {
+                    const uint32_t keep = left != 0;  // all regions restart after a fold
+                    if (left == 0) {
+                        left = min(OZT_FOLD, nk - it);
+                        if (folds > 0 && !mbar_wait_or_abort(mb_free, (folds - 1) & 1, abort_flag)) { ok = false; break; }
+                    }
+                    if (!mbar_wait_or_abort(mb_full + 8 * slot, phase, abort_flag)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    const uint64_t so = (uint64_t)((slot * OZT_STAGE) >> 4);
 #pragma unroll
-        for (int t = 0; t < OZ_S; ++t) {
-            uint32_t r[16];
-            tmem_ld16(tpart + (uint32_t)(t * OZT_BN), r);
+                    for (int p = 0; p < OZ_S; ++p) {
+                        // groups p .. 6 (q = 0 .. 6 - p): consecutive B slices into
+                        // consecutive regions, at most 4 slices (N = 256) per MMA
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                if (t < 5)
-                    acc[j] += (long long)group_int(__uint_as_float(r[j]), 0x1p-12f * (float)(1ull << (8 * t)),
-                                                   (float)(1ull << (8 * t)))
-                              << (32 - 8 * t);
-                else
-                    low[j] += __uint_as_float(r[j]);
-            }
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-        asm volatile("bar.sync 1, %0;\n" ::"n"(OZT_THREADS) : "memory");  // regions free again
-    };
-    if (producer) {
-        // one thread issues the stage copies (one stage image of each operand),
-        // OZT_DIST stages ahead of the fold that follows a stage
-        const size_t nks = (size_t)(Kp / OZT_KC);
-        const __nv_bfloat16 *srcA = As + (size_t)bm * nks * (OZ_S * OZT_BM * OZT_KC);
-        const __nv_bfloat16 *srcB = Bs + (size_t)bn * nks * (OZ_S * OZT_BN * OZT_KC);
-        int issued = 0;  // stages whose copies were issued (all of them unless a wait ran out)
-        for (int st = 0; st < nk + OZT_DIST; ++st) {
-            if (st < nk && tid == OZT_PRODUCER && !*abort_flag) {
-                const int slot = st % OZT_NST;
-                // slot st % NST was last read by the MMAs of stage st - NST
-                if (st >= OZT_NST &&
-                    !mbar_wait_or_abort(mb_empty + 8 * slot, ((st / OZT_NST) - 1) & 1, abort_flag)) {
-                    ok = false;
-                    *abort_flag = 1;
-                }
-            }
-            if (st < nk && tid == OZT_PRODUCER && !*abort_flag) {
-                const int slot = st % OZT_NST;
-                const uint32_t full = mb_full + 8 * slot;
-                mbar_expect_tx(full, (uint32_t)OZT_STAGE);
-                const uint32_t a0 = sbase + (uint32_t)(slot * OZT_STAGE);
-                const uint32_t b0 = a0 + OZ_S * OZT_A_SLICE;
-                const size_t ks = (size_t)(kbeg / OZT_KC + st);
-                bulk_load(a0, srcA + ks * (OZ_S * OZT_BM * OZT_KC), (uint32_t)(OZ_S * OZT_A_SLICE), full);
-                bulk_load(b0, srcB + ks * (OZ_S * OZT_BN * OZT_KC), (uint32_t)(OZ_S * OZT_B_SLICE), full);
-                issued = st + 1;
-            }
-            __syncwarp();
-            const int done = st - OZT_DIST;
-            if (done >= 0 && is_fold(done)) fold_part();
-        }
-        // every copy that was issued has landed before the CTA leaves (waits
-        // bounded; the last issued stage of each slot is its latest phase)
-        if (tid == OZT_PRODUCER)
-            for (int st = max(0, issued - OZT_NST); st < issued; ++st)
-                ok = mbar_wait(mb_full + 8 * (st % OZT_NST), (st / OZT_NST) & 1) && ok;
-        __syncwarp();
-    } else {
-        for (int it = 0; it < nk; ++it) {
-            if (tid == 0) {
-                const int slot = it % OZT_NST;
-                bool go = !*abort_flag;
-                if (go && !mbar_wait_or_abort(mb_full + 8 * slot, (it / OZT_NST) & 1, abort_flag)) {
-                    ok = false;
-                    *abort_flag = 1;
-                    go = false;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t a0 = sbase + (uint32_t)(slot * OZT_STAGE);
-                const uint32_t b0 = a0 + OZ_S * OZT_A_SLICE;
-                const uint32_t keep = (it % OZT_FOLD) == 0 ? 0u : 1u;  // all regions restart after a fold
-#pragma unroll
-                for (int p = 0; p < OZ_S; ++p) {
-                    if (!go) break;  // no MMA on a stage whose copies did not land
-                    const uint64_t ad = umma_desc(a0 + p * OZT_A_SLICE, OZT_LBO_A);
-                    // groups p .. 6 (q = 0 .. 6 - p): consecutive B slices into
-                    // consecutive regions, at most 4 slices (N = 256) per MMA
-#pragma unroll
-                    for (int q0 = 0; q0 <= OZ_S - 1 - p; q0 += 4) {
-                        const int nq = min(4, OZ_S - p - q0);
-                        umma_bf16(tmem + (uint32_t)((p + q0) * OZT_BN), ad, umma_desc(b0 + q0 * OZT_BN * 16, OZT_LBO_B),
-                                  umma_idesc(nq * OZT_BN), p == 0 ? keep : 1u);
+                        for (int q0 = 0; q0 <= OZ_S - 1 - p; q0 += 4) {
+                            const int nq = min(4, OZ_S - p - q0);
+                            umma_bf16(tmem + (uint32_t)((p + q0) * OZT_BN), da + so + ((p * OZT_A_SLICE) >> 4),
+                                      db + so + ((q0 * OZT_BN * 16) >> 4), umma_idesc(nq * OZT_BN), p == 0 ? keep : 1u);
+                        }
+                    }
+                    umma_commit(mb_empty + 8 * slot);
+                    if (--left == 0) {
+                        umma_commit(mb_fold);
+                        ++folds;
+                    }
+                    if (++slot == OZT_NST) {
+                        slot = 0;
+                        phase ^= 1;
                     }
                 }
-                // committed whether or not MMAs were issued: the slot and the
-                // fold barrier complete once every earlier MMA has finished
-                umma_commit(mb_empty + 8 * slot);
-                if (is_fold(it)) umma_commit(mb_fold);
             }
-            __syncwarp();
-            if (is_fold(it)) fold_part();
+            umma_commit(mb_done);
+            ok = mbar_wait(mb_done, 0) && ok;
+        }
+        __syncwarp();
+    } else if (warp == OZT_FOLDERS / 32 + 1) {  // ---- the copies
+        if (lane == 0) {
+            const size_t nks = (size_t)(Kp / OZT_KC);
+            int issued = 0;  // stages whose copies were issued (all of them unless a wait ran out)
+            for (int w = blockIdx.x; ok && w < items; w += gridDim.x) {
+                int sp, bm, bn;
+                ozt_item(w, tiles, nbm, nbn, halfN_tiles, upper_only, sp, bm, bn);
+                const int nk = stages(sp);
+                const size_t k0 = (size_t)(sp * kchunk / OZT_KC);
+                const __nv_bfloat16 *srcA = As + ((size_t)bm * nks + k0) * (OZ_S * OZT_BM * OZT_KC);
+                const __nv_bfloat16 *srcB = Bs + ((size_t)bn * nks + k0) * (OZ_S * OZT_BN * OZT_KC);
+                for (int st = 0; st < nk; ++st) {
+                    const int slot = issued % OZT_NST;
+                    // the slot was last read by the MMAs of stage issued - NST
+                    if (issued >= OZT_NST &&
+                        !mbar_wait_or_abort(mb_empty + 8 * slot, ((issued / OZT_NST) - 1) & 1, abort_flag)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t full = mb_full + 8 * slot;
+                    mbar_expect_tx(full, (uint32_t)OZT_STAGE);
+                    const uint32_t a0 = sbase + (uint32_t)(slot * OZT_STAGE);
+                    const uint32_t b0 = a0 + OZ_S * OZT_A_SLICE;
+                    bulk_load(a0, srcA + (size_t)st * (OZ_S * OZT_BM * OZT_KC), (uint32_t)(OZ_S * OZT_A_SLICE), full);
+                    bulk_load(b0, srcB + (size_t)st * (OZ_S * OZT_BN * OZT_KC), (uint32_t)(OZ_S * OZT_B_SLICE), full);
+                    ++issued;
+                }
+            }
+            // every copy that was issued has landed before the CTA leaves (waits
+            // bounded; the last issued stage of each slot is its latest phase)
+            for (int st = max(0, issued - OZT_NST); st < issued; ++st)
+                ok = mbar_wait(mb_full + 8 * (st % OZT_NST), (st / OZT_NST) & 1) && ok;
+        }
+        __syncwarp();
+    } else {  // ---- folds and results
+        const int lrow = 32 * (warp & 3) + lane, lcol = OZT_CPT * (warp >> 2);
+        const uint32_t tpart = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)lcol;
+        int folds = 0;
+        for (int w = blockIdx.x; w < items; w += gridDim.x) {
+            int sp, bm, bn;
+            ozt_item(w, tiles, nbm, nbn, halfN_tiles, upper_only, sp, bm, bn);
+            long long acc[OZT_CPT];
+            float low[OZT_CPT];
+#pragma unroll
+            for (int c = 0; c < OZT_CPT; ++c) {
+                acc[c] = 0;
+                low[c] = 0.f;
+            }
+            for (int nk = stages(sp); nk > 0; nk -= OZT_FOLD) {
+                ok = __all_sync(0xffffffffu, mbar_wait_or_abort(mb_fold, folds & 1, abort_flag));
+                if (!ok) break;
+                ++folds;
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                static_assert(OZT_CPT == 16, "one 16-column TMEM load per region");
+#pragma unroll
+                for (int t = 0; t < OZ_S; ++t) {
+                    uint32_t r[16];
+                    tmem_ld16(tpart + (uint32_t)(t * OZT_BN), r);
+                    if (t == OZ_S - 1) {  // regions free again
+                        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                        if (lane == 0)
+                            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mb_free) : "memory");
+                    }
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        if (t < 5)
+                            acc[j] += (long long)group_int(__uint_as_float(r[j]), 0x1p-12f * (float)(1ull << (8 * t)),
+                                                           (float)(1ull << (8 * t)))
+                                      << (32 - 8 * t);
+                        else
+                            low[j] += __uint_as_float(r[j]);
+                    }
+                }
+            }
+            if (!ok) break;
+            const int i = bm * OZT_BM + lrow, j0 = bn * OZT_BN + lcol;
+            const int ea = Ea[i] - 2090;
+            if (W) {
+                double2 *wp = reinterpret_cast<double2 *>(W + (size_t)sp * Mp * Np + (size_t)i * Np + j0);
+#pragma unroll
+                for (int c = 0; c < OZT_CPT; c += 2)
+                    wp[c / 2] = make_double2(oz_value(acc[c], low[c], ea + Eb[j0 + c]),
+                                             oz_value(acc[c + 1], low[c + 1], ea + Eb[j0 + c + 1]));
+                continue;
+            }
+            if (i >= M) continue;
+#pragma unroll
+            for (int c0 = 0; c0 < OZT_CPT; c0 += 8) {  // the reads of C ahead of its writes
+                double old[8];
+                double *cp[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const int jj = j0 + c0 + c, part = jj >= H, j = jj - part * H;
+                    cp[c] = j < N ? reinterpret_cast<double *>(C + (int64_t)j * ldc + i) + part : nullptr;
+                    old[c] = cp[c] && beta != 0.0 ? *cp[c] : 0.0;
+                }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const double v = oz_value(acc[c0 + c], low[c0 + c], ea + Eb[j0 + c0 + c]);
+                    double r = alpha == 1.0 ? v : alpha * v;
+                    if (beta != 0.0) r = fma(beta, old[c], r);
+                    if (cp[c]) *cp[c] = r;
+                }
+            }
         }
     }
     if (!ok && lane == 0) atomicAdd(status, 1u);
-
-    const int i = m0 + lrow;
-    const int ea = Ea[i];
-#pragma unroll
-    for (int c = 0; c < OZT_CPT; ++c) {
-        const int jj = n0 + lcol + c;
-        const double v = oz_value(acc[c], low[c], ea + Eb[jj] - 2090);
-        const int part = jj >= H, j = jj - part * H;
-        if (W) {
-            W[(size_t)sp * Mp * Np + (size_t)i * Np + jj] = v;
-        } else if (i < M && j < N) {
-            double *cp = reinterpret_cast<double *>(C + (int64_t)j * ldc + i) + part;
-            double r = alpha == 1.0 ? v : alpha * v;
-            if (beta != 0.0) r = fma(beta, *cp, r);
-            *cp = r;
-        }
-    }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
@@ -973,6 +1027,9 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
         e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM);
     else
         e = cudaFuncSetAttribute(oz_gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZT_SMEM);
+    int dev = 0, nsm = 152;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     char *w = static_cast<char *>(ws);
     __nv_bfloat16 *As = reinterpret_cast<__nv_bfloat16 *>(w);
@@ -1026,7 +1083,9 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const unsigned tm = (unsigned)(p.Mp / bm), tn = (unsigned)(p.Np / OZ_BN);
-        const dim3 grid = legacy ? dim3(tm, tn, (unsigned)p.splits) : dim3(tm * tn, 1, (unsigned)p.splits);
+        const int64_t tiles = tile_count(p.Mp, p.Np, bm, upper, halfN_tiles), items = tiles * p.splits;
+        if (!legacy && items > INT_MAX) return cudaErrorInvalidValue;
+        const dim3 grid = legacy ? dim3(tm, tn, (unsigned)p.splits) : dim3((unsigned)std::min<int64_t>(items, nsm));
         cudaEvent_t ev1 = nullptr;
         if (timer) {
             cudaEvent_t ev0;
@@ -1041,7 +1100,7 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
         else
             oz_gemm_tc_kernel<<<grid, OZT_THREADS, OZT_SMEM, s>>>(As, Bs, Ea, Eb, Wp, C, ldc, M, N, H,
                                                                  (int)p.Mp, (int)p.Np, (int)p.Kp,
-                                                                 (int)p.kchunk, halfN_tiles,
+                                                                 (int)p.kchunk, (int)tiles, (int)items, halfN_tiles,
                                                                  upper ? 1 : 0, alpha, b, status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (timer && (e = cudaEventRecord(ev1, s)) != cudaSuccess) return e;
