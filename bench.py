@@ -466,7 +466,7 @@ def run_ours(a, rank, world, local):
     lu_avg = statistics.mean(lu_ms)
     achieved = lu_flops / (lu_avg / 1e3) / 1e12
     ldab = 2 * kl + ku + 32
-    roof_lu = {"bound": "alu", "kernel": "band_lu_cluster_kernel<float2> (complex64, two-CTA cluster per point)",
+    roof_lu = {"bound": "alu", "kernel": "band_lu_kernel<float2> (complex64, a cluster of CTAs per point)",
                "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                "frac": achieved / FP32_PEAK_TFLOPS,
                "traffic": traffic_lu,
@@ -490,10 +490,10 @@ def run_ours(a, rank, world, local):
                              "(the ||T(z_j)|| kernel + the assembly), so the fraction is a lower bound"}
 
     # first solve of all points: the complex64 factors streamed once per 16
-    # right-hand sides (two CTAs per point), against the copy bandwidth
+    # right-hand sides, against the copy bandwidth
     solve_avg = statistics.mean(solve_ms)
     solve_bytes = 8.0 * ldab * n * p.N
-    roof_solve = {"bound": "hbm", "kernel": "band_solve2_kernel<float2> (streaming banded solve, first solve)",
+    roof_solve = {"bound": "hbm", "kernel": "band_solve_stream_kernel<float2> (streaming banded solve, first solve)",
                   "achieved": solve_bytes / (solve_avg / 1e3) / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                   "frac": solve_bytes / (solve_avg / 1e3) / 1e9 / peaks["hbm_gbs"], "hbm_frac":
                   solve_bytes / (solve_avg / 1e3) / 1e9 / peaks["hbm_gbs"], "traffic": traffic_solve,

@@ -219,7 +219,7 @@ enum { RSRR_GEMM_AUTO = 0, RSRR_GEMM_FP64 = 1, RSRR_GEMM_OZAKI = 2, RSRR_GEMM_OZ
  * streaming solve; same arithmetic, kept for comparison and as the fallback
  * for bands too wide for the streaming solve's shared-memory window. */
 /* RSRR_FLAG_ONE_CTA_LU: band LU of rsrr_sample by one CTA per sampling point
- * instead of a cluster of two CTAs per point (the second CTA updates most of
+ * instead of a cluster of up to eight CTAs per point (the others update most of
  * the trailing window while the first factors the next panel); the factors
  * are bitwise the same, the flag exists for comparison. */
 /* RSRR_FLAG_INJECT_TIMEOUT: failure detection without a GPU fault.
@@ -279,7 +279,7 @@ enum {
  * refinement sweep).  If capture is not possible the call runs eagerly.
  * rsrr_add_points drops the graph (buffers move).
  * RSRR_FLAG_AUTOTUNE: the first rsrr_sample of the band path times the band
- * LU as a cluster of two CTAs per point and as one CTA per point, and the
+ * LU as a cluster of CTAs per point and as one CTA per point, and the
  * streaming and the one-kernel solve, on the handle's own data, keeps the
  * faster of each (results agree: the LU variants bitwise, the solves to
  * rounding before refinement) and caches the choice per shape (n, kl, ku, N,

@@ -1273,7 +1273,7 @@ std::mutex g_tune_mu;
 std::map<TuneKey, TuneVal> g_tune;
 }  // namespace
 
-// Times the band LU variants (cluster of two CTAs, one CTA per point; same
+// Times the band LU variants (a cluster of CTAs, one CTA per point; same
 // factors bit for bit) and the solve variants (streaming, one-kernel) on the
 // handle's own problem, keeps the faster of each, and caches the choice.
 rsrr_status Handle::autotune(cudaStream_t s) {

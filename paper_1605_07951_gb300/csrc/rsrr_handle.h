@@ -106,7 +106,7 @@ struct Handle {
     size_t gmres_bytes = 0;
     bool solve2 = false;              // streaming band solve possible (block permutations allocated)
     bool use_solve2 = false;          // streaming band solve in use (autotuned or solve2)
-    bool cluster_lu = true;           // band LU by a cluster of two CTAs per point
+    bool cluster_lu = true;           // band LU by a cluster of CTAs per point
     bool tuned = false;               // the autotuner's choice is applied
     // CUDA graph of rsrr_sample (RSRR_FLAG_GRAPH, band path)
     cudaGraph_t graph = nullptr;

@@ -54,8 +54,8 @@ template <typename C>
 cudaError_t launch_assemble(C *ab, const BandGeom &g, const DevProblem &p, cudaStream_t s);
 cudaError_t launch_tnorm(double *tnorm, const DevProblem &p, cudaStream_t s);
 // dinv: per point and NB block, L11^{-1} then U11^{-1} (NB x NB each)
-// cluster: two CTAs per point with one-panel lookahead (band_lu.cu); the
-// factors are bitwise those of the one-CTA kernel
+// cluster: up to eight CTAs per point (band_lu.cu picks how many from the band and the
+// number of points); the factors are bitwise those of one CTA per point
 cudaError_t launch_band_lu_c64(float2 *ab, int32_t *piv, int32_t *info, float2 *dinv,
                                const BandGeom &g, int N, int n, cudaStream_t s, bool cluster = false);
 cudaError_t launch_band_lu_c128(double2 *ab, int32_t *piv, int32_t *info, double2 *dinv,
