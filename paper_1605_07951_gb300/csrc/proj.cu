@@ -185,7 +185,7 @@ struct Gemm {
         const int64_t tiles = hermitian ? (int64_t)tm * (tm + 1) / 2 : (int64_t)tm * tn;
         // splits of K that fill whole waves of SMs (the FP64 unit of an SM is
         // shared by its CTAs, so a wave costs its depth).  Below the line of the
-        // sliced products, the 16 products of an SS-RR solve of order 3600: 12.0
+        // sliced products, the 16 products of an RSRR solve of order 3600: 12.0
         // -> 6.6 ms, where two CTAs an SM and at most K / 256 splits stood before
         // and every tile had 64 columns
         int splits = 1;
@@ -479,7 +479,7 @@ RSRR_DEV Rot rot_of(const double2 *__restrict__ H, int k, int p, int q) {
 // (one per pair, from the old matrix) into shared memory `srot`.  Only the blocks
 // a <= b are computed, the others are their conjugates; an element of a block to
 // a thread, since the FP64 unit charges for a warp's instructions and not for its
-// lanes.  The two decompositions of an SS-RR solve of order 3600: 9.7 -> 4.8 ms, of
+// lanes.  The two decompositions of an RSRR solve of order 3600: 9.7 -> 4.8 ms, of
 // order 40000: 17.0 -> 8.8 ms (with the barrier of one atomic above).
 RSRR_DEV void jacobi_round(const double2 *__restrict__ Hold, double2 *__restrict__ Hnew,
                            double2 *__restrict__ Y, int k, int kp, int r, Rot *__restrict__ srot) {
