@@ -142,6 +142,7 @@ public:
         for (auto &t : pool_) t.join();
     }
     void run(int count, const std::function<void(int, int)> &fn) {
+        if (count <= 0) return;  // behind the last column of a step there is nothing, not even an address
         const int n = (int)pool_.size() + 1;
         if (n == 1) {
             fn(0, count);
