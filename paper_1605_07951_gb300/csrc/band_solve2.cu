@@ -454,11 +454,17 @@ cudaError_t launch_block_perm(int32_t *bperm, const int32_t *piv, int n, int kl,
 // multiple of the block size so that the NB rows of a block never wrap around
 static int sv_window(const BandGeom &g, int nb) { return (g.kl + g.ku + 2 * nb + nb - 1) / nb * nb; }
 
-// Bands for which the streaming solve is taken: the widest shape has room for
-// three units of 128 rows beside its window (kl + ku up to about 560 in
-// complex64); wider ones take the one-kernel solve.
+// Bands for which the streaming solve is taken: a window without its padding
+// columns and three units of 128 rows fit in shared memory, for the widest shape
+// (kl + ku up to 576 in complex64, 736 in complex128, 2272 and 2352 in their real
+// counterparts); wider ones take the one-kernel solve.  At the line (half-bandwidth
+// 288, n = 6000, 64 points, 32 right-hand sides) a first solve takes 2.6 ms here and
+// 12.4 ms there, a whole refined sampling 154 and 173 ms.  The launch needs less
+// than this line asks for (sv_launch: down to two units of 32 rows).
 template <typename C, int NB, int LC> static size_t sv_need(const BandGeom &g) {
-    return SvLayout<C, NB, LC>::smem((g.kl + g.ku + 3 * NB + NB - 1) / NB * NB, 128, 3);
+    using LY = SvLayout<C, NB, LC>;
+    const int WR = (g.kl + g.ku + 3 * NB + NB - 1) / NB * NB;
+    return LY::smem(WR, 128, 3) - LY::w_bytes(WR) + sizeof(C) * (size_t)WR * (LC + 1);
 }
 size_t band_solve2_smem_c64(const BandGeom &g) { return sv_need<float2, NB_C64, 16>(g); }
 size_t band_solve2_smem_c128(const BandGeom &g) { return sv_need<double2, NB_C128, 8>(g); }
