@@ -7,9 +7,12 @@
 // g = M W0 Sigma0^{-1} b with M = [A_0 .. A_{K-1}].
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cmath>
 #include <complex>
+#include <condition_variable>
 #include <functional>
+#include <mutex>
 #include <thread>
 #include <vector>
 
@@ -124,7 +127,9 @@ void reflect_columns(cplx *a, int ld, int cols, const cplx *v, int n, double *nr
 
 // Threads of one decomposition, started once: a thread start costs more than most
 // steps.  run(count, fn) calls fn(begin, end) on a contiguous part of 0 .. count - 1
-// per thread; a waiting thread yields, since other solves may share the cores.
+// per thread.  A waiting thread yields for KEEN microseconds, longer than the serial part
+// of a step, and then sleeps: the long serial parts leave the cores to others (16 cores,
+// k = 60 and 237: 3.2 and 96 ms with and without the sleep).
 // (Threads started for every column of the QR, and scalar complex products: the whole
 // solve of an order-3600 problem on 16 cores 46.3 -> 35.2 ms with these and the vector
 // loops above, of order 40000 241 -> 232 ms.)
@@ -138,7 +143,7 @@ public:
     }
     ~Workers() {
         fn_ = nullptr;
-        epoch_.fetch_add(1, std::memory_order_release);
+        publish();
         for (auto &t : pool_) t.join();
     }
     void run(int count, const std::function<void(int, int)> &fn) {
@@ -152,17 +157,35 @@ public:
         part_ = ((count + n - 1) / n + 3) / 4 * 4;
         count_ = count;
         left_.store(n - 1, std::memory_order_relaxed);
-        epoch_.fetch_add(1, std::memory_order_release);
+        publish();
         fn(0, std::min(part_, count));
         while (left_.load(std::memory_order_acquire) > 0) std::this_thread::yield();
     }
 
 private:
+    static constexpr int KEEN = 2000;
+    void publish() {
+        epoch_.fetch_add(1);
+        if (asleep_.load() == 0) return;  // a thread that counts itself later sees this epoch first
+        { std::lock_guard<std::mutex> lk(mu_); }
+        cv_.notify_all();
+    }
+    unsigned next(unsigned seen) {
+        const auto until = std::chrono::steady_clock::now() + std::chrono::microseconds(KEEN);
+        do {
+            const unsigned e = epoch_.load(std::memory_order_acquire);
+            if (e != seen) return e;
+            std::this_thread::yield();
+        } while (std::chrono::steady_clock::now() < until);
+        std::unique_lock<std::mutex> lk(mu_);
+        asleep_.fetch_add(1);
+        cv_.wait(lk, [&]() { return epoch_.load() != seen; });
+        asleep_.fetch_sub(1);
+        return epoch_.load();
+    }
     void loop(int w) {
         for (unsigned seen = 0;;) {
-            unsigned e;
-            while ((e = epoch_.load(std::memory_order_acquire)) == seen) std::this_thread::yield();
-            seen = e;
+            seen = next(seen);
             if (!fn_) return;
             const int b = std::min(count_, w * part_), t = std::min(count_, b + part_);
             if (b < t) (*fn_)(b, t);
@@ -171,9 +194,11 @@ private:
     }
     std::vector<std::thread> pool_;
     std::atomic<unsigned> epoch_{0};
-    std::atomic<int> left_{0};
+    std::atomic<int> left_{0}, asleep_{0};
     const std::function<void(int, int)> *fn_ = nullptr;
     int part_ = 0, count_ = 0;
+    std::mutex mu_;
+    std::condition_variable cv_;
 };
 
 // Truncated SVD A = U S W^H of A (r x c) through a column-pivoted Householder
