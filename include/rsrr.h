@@ -559,9 +559,10 @@ rsrr_status rsrr_solve_band_noalloc(int64_t n, int32_t kl, int32_t ku, const rsr
  *   stream     work is queued on it; the call waits for it before returning
  * Work space comes from a pool of the library, which keeps at most 2 GiB of it
  * on the device between calls and gives that back when a handle or a server is
- * created; it does not survive a cudaDeviceReset.  Returns OK, EINVAL,
- * ENOMEM (work space), ETIMEOUT (a bounded wait of the tensor-core kernel ran
- * out) or ECUDA; the message is in rsrr_last_error(NULL). */
+ * created; the driver gives it to any allocation of the process that does not
+ * fit beside it.  The entry point works on after a cudaDeviceReset.  Returns OK,
+ * EINVAL, ENOMEM (work space), ETIMEOUT (a bounded wait of the tensor-core kernel
+ * ran out) or ECUDA; the message is in rsrr_last_error(NULL). */
 rsrr_status rsrr_zgemm(int32_t M, int32_t N, int32_t K, int32_t conjA, const rsrr_c128 *A,
                        int64_t lda, const rsrr_c128 *B, int64_t ldb, rsrr_c128 *C, int64_t ldc,
                        double alpha, double beta, int32_t method, int32_t hermitian,

@@ -1131,7 +1131,9 @@ std::string &thread_error();  // api.cu: last error of a handle-less call
 // 40000 x 500 Gram matrix's 3.4); allocations and frees are ordered on the
 // caller's stream, so threads and streams do not share a block in use.  What is
 // kept is given back when a handle or a server is created, and when an
-// allocation of the pool fails.
+// allocation of the pool fails; the driver takes it back by itself for any other
+// allocation that does not fit beside it.  A pool is not among what a
+// cudaDeviceReset destroys: it serves the next context as before.
 constexpr uint64_t ZGEMM_KEEP = 2ull << 30;
 constexpr int ZGEMM_DEVICES = 64;
 static std::mutex g_zgemm_mu;
