@@ -723,7 +723,7 @@ size_t Handle::estimate_bytes() {
     dry = false;
     size_t b = device_bytes;
     device_bytes = 0;
-    b += projection_ws_bytes(N * L, n, m);
+    b += projection_ws_bytes(*this);
     // (composite Gauss on a rectangle rounds each side to whole panels: up to
     // two more panels of 10 nodes than N_Q)
     const int nq = region.kind == RSRR_REGION_RECT ? std::max(opts.NQ + 20, 40) : opts.NQ;

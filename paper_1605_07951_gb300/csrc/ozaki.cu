@@ -964,14 +964,17 @@ int64_t tile_count(int64_t Mp, int64_t Np, int bm, bool upper, int64_t halfN) {
     return t;
 }
 
-OzPlan make_plan(int M, int N, int K, bool hermitian, size_t ws_bytes, int bm, int64_t kmax = OZ_KMAX) {
+OzPlan make_plan(int M, int N, int K, bool hermitian, size_t ws_bytes, int bm, int64_t kmax = OZ_KMAX,
+                 bool packed = false) {
     OzPlan p{};
     p.Mp = rup(M, bm);
     // a Hermitian result's halves start on tiles of their own, so that the tiles
-    // below the diagonal of both can be left out
-    p.H = hermitian ? rup(N, OZ_BN) : N;
+    // below the diagonal of both can be left out (packed: they do not, for
+    // ozaki_padding_bytes)
+    p.H = hermitian && !packed ? rup(N, OZ_BN) : N;
     p.Np = rup(2 * p.H, OZ_BN);
-    const int64_t tiles = tile_count(p.Mp, p.Np, bm, hermitian, hermitian ? p.H / OZ_BN : p.Np / OZ_BN);
+    const int64_t tiles = packed ? (p.Mp / bm) * (p.Np / OZ_BN) / 2
+                                 : tile_count(p.Mp, p.Np, bm, hermitian, hermitian ? p.H / OZ_BN : p.Np / OZ_BN);
     const int64_t Kall = std::max(K, 1);
     auto fit = [&](int64_t kc) {
         p.Kc = kc;
@@ -990,10 +993,17 @@ OzPlan make_plan(int M, int N, int K, bool hermitian, size_t ws_bytes, int bm, i
 }
 }  // namespace
 
-size_t ozaki_workspace_bytes(int M, int N, int K, bool hermitian, int64_t kmax) {
+static size_t planned_bytes(int M, int N, int K, bool hermitian, int64_t kmax, bool packed) {
     if (kmax <= 0 || kmax > OZ_KMAX) kmax = OZ_KMAX;
-    return std::max(make_plan(M, N, K, hermitian, SIZE_MAX, OZ_BM, kmax).bytes,
-                    make_plan(M, N, K, hermitian, SIZE_MAX, OZT_BM, kmax).bytes);
+    return std::max(make_plan(M, N, K, hermitian, SIZE_MAX, OZ_BM, kmax, packed).bytes,
+                    make_plan(M, N, K, hermitian, SIZE_MAX, OZT_BM, kmax, packed).bytes);
+}
+size_t ozaki_workspace_bytes(int M, int N, int K, bool hermitian, int64_t kmax) {
+    return planned_bytes(M, N, K, hermitian, kmax, false);
+}
+size_t ozaki_padding_bytes(int N, int K, int64_t kmax) {
+    const size_t padded = planned_bytes(N, N, K, true, kmax, false), packed = planned_bytes(N, N, K, true, kmax, true);
+    return padded > packed ? padded - packed : 0;
 }
 
 double ozaki_tc_flops(int M, int N, int K, bool hermitian, bool legacy) {

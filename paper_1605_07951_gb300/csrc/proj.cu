@@ -862,13 +862,36 @@ __global__ void scatter_inverse_fill_kernel(double2 *__restrict__ X, const doubl
 // Work space of the sliced products: the Gram matrix of the n x NL block in
 // chunks of at most 32768 of its depth (the other products of the sparse kind
 // need less), capped at 8 GiB; a product that needs more runs in more chunks.
-static size_t ozaki_ws_bytes(int NL, int64_t n) {
-    const int nc = (int)std::min<int64_t>(n, INT32_MAX / 2);
-    return std::min(ozaki_workspace_bytes(NL, NL, nc, true, 32768), (size_t)8 << 30);
+// None where every product runs in FP64.
+constexpr int64_t GRAM_CHUNK = 32768;
+static size_t ozaki_ws_bytes(const Handle &h) {
+    if (h.opts.gemm == RSRR_GEMM_FP64) return 0;
+    const int NL = h.N * h.L, nc = (int)std::min<int64_t>(h.n, INT32_MAX / 2);
+    return std::min(ozaki_workspace_bytes(NL, NL, nc, true, GRAM_CHUNK), (size_t)8 << 30);
+}
+
+// Elements of the split-K slabs (splits x M x N) of the FP64 products: four NL x NL
+// slabs or 8 M elements (with more the last wave of blocks is a few percent of a
+// product).  Where the large products are sliced, the slabs make room for what the
+// later layouts add to a handle, so that it fits the budgets it has fitted: the
+// padding of the slices, four ints a block in the records of the band solve, the
+// second set of SS-FULL's node weights.  The products left to FP64 then have M N K <
+// 2^27 (Hermitian M M K < 2^28) and at most K / 64 splits: 2^22 elements serve them.
+static size_t split_elems(const Handle &h) {
+    const size_t NL = (size_t)h.N * h.L, full = std::max<size_t>(NL * NL * 4, (size_t)8 << 20);
+    if (h.opts.gemm == RSRR_GEMM_FP64) return full;
+    const int nc = (int)std::min<int64_t>(h.n, INT32_MAX / 2);
+    size_t added = ozaki_padding_bytes((int)NL, nc, GRAM_CHUNK);
+    if (h.solve2) added += (size_t)h.fcap * ((h.n + h.geom.nb - 1) / h.geom.nb) * 4 * sizeof(int32_t);
+    added += sizeof(double2) * 2 * (size_t)std::max(h.opts.KQ, 1) * (std::max(h.opts.NQ, 20) + 20) + 256;
+    const size_t least = (size_t)1 << 22, take = (added + sizeof(double2) - 1) / sizeof(double2) + 16;
+    return std::max(least, full - std::min(full, take));
 }
 
 // Workspace layout of the projection stage (carved from one allocation).
-static void carve_ws(char *cp, ProjWs &ws, int NL, int64_t n, int terms) {
+static void carve_ws(char *cp, ProjWs &ws, const Handle &h) {
+    const int NL = h.N * h.L, terms = h.m;
+    const int64_t n = h.n;
     const size_t NL2 = (size_t)NL * NL;
     ws.norms = carve<double>(cp, NL);
     ws.G = carve<double2>(cp, NL2);
@@ -889,25 +912,21 @@ static void carve_ws(char *cp, ProjWs &ws, int NL, int64_t n, int terms) {
     ws.jacc = carve<double>(cp, 2 * 4096);
     ws.Q1 = carve<double2>(cp, (size_t)n * NL);
     ws.Ytmp = carve<double2>(cp, (size_t)n * NL);
-    // (split-K slabs of the FP64 products; less than a round size by what the
-    // sliced products' padded halves and the block records of the band solve add)
-    ws.gws_elems = std::max<size_t>(NL2 * 4, (size_t)8 << 20) - (NL % 64 ? (size_t)9 << 19 : (size_t)1 << 20);
+    ws.gws_elems = split_elems(h);
     ws.gws = carve<double2>(cp, ws.gws_elems);
-    ws.ows_bytes = ozaki_ws_bytes(NL, n);
+    ws.ows_bytes = ozaki_ws_bytes(h);
     ws.ows = carve<char>(cp, ws.ows_bytes);
     ws.Qall = carve<double2>(cp, (size_t)n * NL);
     ws.P = carve<double2>(cp, (size_t)std::max(terms, RSRR_MAX_TERMS) * NL2);
     ws.end = cp;
 }
 
-static size_t ws_bytes(int NL, int64_t n, int terms) {
+size_t projection_ws_bytes(const Handle &h) {
     ProjWs ws;
     char *base = reinterpret_cast<char *>((uintptr_t)0);
-    carve_ws(base, ws, NL, n, terms);
+    carve_ws(base, ws, h);
     return (size_t)(ws.end - base);
 }
-
-size_t projection_ws_bytes(int NL, int64_t n, int terms) { return ws_bytes(NL, n, terms); }
 
 // Orthonormal basis of the dominant singular subspace of Sn = X D^{-1}:
 // deflated multi-level Gram.  Level l works on the remainder R_l (R_0 = Sn):
@@ -928,7 +947,7 @@ rsrr_status Handle::project(cudaStream_t s) {
     // columns of the matrix whose basis is taken: S (N L) or the moments M (K L)
     const int nc = opts.method == RSRR_METHOD_SSRR_M ? opts.K * L : NL;
     if (!proj_ws) {
-        const size_t bytes = ws_bytes(NL, nn, m);
+        const size_t bytes = projection_ws_bytes(*this);
         void *p = nullptr;
         cudaError_t e = raw_alloc(&p, bytes);
         if (e != cudaSuccess) return fail(RSRR_ENOMEM, "projection work space", e);
@@ -936,7 +955,7 @@ rsrr_status Handle::project(cudaStream_t s) {
         proj_ws_bytes = bytes;
     }
     ProjWs ws;
-    carve_ws(reinterpret_cast<char *>(proj_ws), ws, NL, nn, m);
+    carve_ws(reinterpret_cast<char *>(proj_ws), ws, *this);
     d_Q = ws.Qall;
     d_P = ws.P;
     Gemm gm;
@@ -1254,7 +1273,7 @@ rsrr_status Handle::ss_ri(cudaStream_t s, std::vector<std::complex<double>> &lam
     using cplx = std::complex<double>;
     const int NL = N * L, K = opts.K;
     if (!proj_ws) {
-        const size_t bytes = ws_bytes(NL, n, m);
+        const size_t bytes = projection_ws_bytes(*this);
         void *p = nullptr;
         cudaError_t e = raw_alloc(&p, bytes);
         if (e != cudaSuccess) return fail(RSRR_ENOMEM, "SS-RI work space", e);
@@ -1262,7 +1281,7 @@ rsrr_status Handle::ss_ri(cudaStream_t s, std::vector<std::complex<double>> &lam
         proj_ws_bytes = bytes;
     }
     ProjWs ws;
-    carve_ws(reinterpret_cast<char *>(proj_ws), ws, NL, n, m);
+    carve_ws(reinterpret_cast<char *>(proj_ws), ws, *this);
     Gemm gm;
     gm.ws = ws.gws;
     gm.ws_elems = ws.gws_elems;
@@ -1357,7 +1376,7 @@ rsrr_status Handle::solve(rsrr_result *out) {
     }
     // v = B g on the GPU
     ProjWs ws;
-    carve_ws(reinterpret_cast<char *>(proj_ws), ws, NL, n, m);
+    carve_ws(reinterpret_cast<char *>(proj_ws), ws, *this);
     Gemm gm;
     gm.ws = ws.gws;
     gm.ws_elems = ws.gws_elems;

@@ -17,7 +17,7 @@ struct Handle;
 rsrr_status prepare(const rsrr_nep *nep, const rsrr_region *region, int32_t N, int32_t L,
                     const rsrr_opts *opts, Handle **out);
 // bytes of the projection stage's work space (proj.cu)
-size_t projection_ws_bytes(int NL, int64_t n, int terms);
+size_t projection_ws_bytes(const Handle &h);
 // SS-FULL moments on the GPU (ssfull_dev.cu): node chunks hold T_Q and its
 // inverse for at most this many bytes; device bytes of the stage for basis k
 constexpr size_t kSsfullChunkBytes = (size_t)1 << 30;

@@ -232,6 +232,8 @@ cudaError_t ozaki_zgemm(int M, int N, int K, bool conjA, const double2 *A, int64
 // gives the work space that rsrr_zgemm keeps on the current device back
 void zgemm_release_kept();
 size_t ozaki_workspace_bytes(int M, int N, int K, bool hermitian, int64_t kmax = 0);
+// what the padding of the two halves of a Hermitian product adds to it
+size_t ozaki_padding_bytes(int N, int K, int64_t kmax);
 // one thread waits, with the tcgen05 kernel's bounded mbarrier wait, on a
 // barrier that nothing completes; after `limit` polls the wait is counted in
 // *status (failure detection without a GPU fault)
