@@ -297,10 +297,11 @@ band_solve_kernel(const C *__restrict__ ab_all, const int32_t *__restrict__ piv_
 // --------------------------------------------------------------------------
 constexpr int RES_LCH = 8;
 
-// (a NaN sorts below every number, as fmax drops it, and comes back when there is nothing else)
+// (a NaN, of either sign, sorts above every number: a column that holds one has no
+// backward error)
 RSRR_DEV long long res_key(double v) {
     const long long b = __double_as_longlong(v);
-    return b > 0x7ff0000000000000LL ? -1LL : b;
+    return b < 0 ? 0x7fffffffffffffffLL : b;
 }
 
 __global__ void residual_kernel(double2 *__restrict__ R, const double2 *__restrict__ X,
@@ -369,8 +370,7 @@ __global__ void residual_kernel(double2 *__restrict__ R, const double2 *__restri
     for (int off = LEFT / 2; off; off >>= 1) key[0] = max(key[0], __shfl_xor_sync(0xffffffffu, key[0], off));
     const int l = id % RES_LCH;
     if (lane % LEFT == 0 && l0 + l < L) {
-        const double v = key[0] < 0 ? __longlong_as_double(0x7ff8000000000000LL) : __longlong_as_double(key[0]);
-        atomic_max_nonneg((id < RES_LCH ? rmax : xmax) + (size_t)pt * L + l0 + l, sqrt(v));
+        atomic_max_nonneg((id < RES_LCH ? rmax : xmax) + (size_t)pt * L + l0 + l, sqrt(__longlong_as_double(key[0])));
     }
 }
 
@@ -389,7 +389,7 @@ __global__ void eta_kernel(double *__restrict__ eta, int32_t *__restrict__ done,
     __syncthreads();
     for (int l = threadIdx.x; l < L; l += blockDim.x) {
         const double den = tnorm[pt] * xmax[pt * L + l] + umax[l];
-        const double e = den > 0.0 ? rmax[pt * L + l] / den : 0.0;
+        const double r = rmax[pt * L + l], e = den == 0.0 ? 0.0 * r : r / den;  // NaN stays NaN
         eta[pt * L + l] = e;
         if (!(e <= tol)) atomicOr(&s_bad, 1);
     }

@@ -908,25 +908,28 @@ __global__ void dense_colmax_kernel(const double2 *__restrict__ R_all, const dou
     const int l = blockIdx.x, pt = blockIdx.y;
     if (done && done[pt]) return;
     const double2 *R = R_all + ((size_t)pt * L + l) * n, *X = X_all + ((size_t)pt * L + l) * n;
-    double r = 0.0, x = 0.0;
-    // squared moduli, one square root at the end (FP64 pipe)
+    // squared moduli by their bit patterns, one square root at the end (FP64 pipe); as
+    // unsigned numbers the patterns of NaN are the largest: a column that holds one
+    // has no backward error
+    unsigned long long r = 0, x = 0;
+    auto bits = [](double v) { return (unsigned long long)__double_as_longlong(v); };
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const double2 u = R[i], v = X[i];
-        r = fmax(r, fma(u.x, u.x, u.y * u.y));
-        x = fmax(x, fma(v.x, v.x, v.y * v.y));
+        r = max(r, bits(fma(u.x, u.x, u.y * u.y)));
+        x = max(x, bits(fma(v.x, v.x, v.y * v.y)));
     }
     for (int off = 16; off; off >>= 1) {
-        r = fmax(r, shfl_down(r, off));
-        x = fmax(x, shfl_down(x, off));
+        r = max(r, shfl_down(r, off));
+        x = max(x, shfl_down(x, off));
     }
-    __shared__ double wr[32], wx[32];
+    __shared__ unsigned long long wr[32], wx[32];
     if ((threadIdx.x & 31) == 0) { wr[threadIdx.x >> 5] = r; wx[threadIdx.x >> 5] = x; }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) { a = fmax(a, wr[q]); b = fmax(b, wx[q]); }
-        rmax[(size_t)pt * L + l] = sqrt(a);
-        xmax[(size_t)pt * L + l] = sqrt(b);
+        unsigned long long a = 0, b = 0;
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) { a = max(a, wr[q]); b = max(b, wx[q]); }
+        rmax[(size_t)pt * L + l] = sqrt(__longlong_as_double((long long)a));
+        xmax[(size_t)pt * L + l] = sqrt(__longlong_as_double((long long)b));
     }
 }
 
