@@ -663,7 +663,10 @@ dense_gemm_update_kernel(C *__restrict__ A_all, int n, int k0) {
 // product per row of the block used 16 of 32.  500 matrices of order 233: 78.6
 // -> 35.6 ms.  FP32: bound by reading the factor from L2 once per chunk, so the
 // chunks are as wide as leaves one for every SM: n = 2048, 64 right-hand sides,
-// 32 points 16.8 -> 5.4 ms for three solves.
+// 32 points 16.8 -> 5.4 ms for three solves, of which the last returns at once.
+// Since then a block's products are summed from zero (update; a solve 2.7 -> 3.1 ms):
+// subtracted one by one from the row they left 2.4 to 3.5 times the backward error
+// (random matrices of order 1200 and 2048, both precisions).
 template <typename C, int NB, int LC, int TH, bool IDENT>
 __global__ void __launch_bounds__(TH, 512 / TH)
 dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_all,
@@ -734,12 +737,14 @@ dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_
         }
         __syncthreads();
     };
-    // rows r_lo .. r_hi-1 -= A(:, k0 .. k0+jb-1) y
+    // rows r_lo .. r_hi-1 -= A(:, k0 .. k0+jb-1) y: eight products at a time summed from
+    // zero, then a block's sums, so that they round by their own size and the row rounds
+    // once a block
     auto update = [&](int k0, int jb, int r_lo, int r_hi) {
         for (int r = r_lo + tid; r < r_hi; r += TH) {
             C acc[LC];
 #pragma unroll
-            for (int c = 0; c < LC; ++c) acc[c] = c < ncol ? B[cb[c] + r] : czero<C>();
+            for (int c = 0; c < LC; ++c) acc[c] = czero<C>();
             const C *a = A + (size_t)k0 * n + r;
             if (jb == NB) {
 #pragma unroll 1
@@ -748,20 +753,23 @@ dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_
 #pragma unroll
                     for (int t = 0; t < 8; ++t) l[t] = a[(size_t)(t0 + t) * n];
 #pragma unroll
-                    for (int t = 0; t < 8; ++t)
+                    for (int c = 0; c < LC; ++c) {
+                        C s = czero<C>();
 #pragma unroll
-                        for (int c = 0; c < LC; ++c) acc[c] = cfms(acc[c], l[t], s_y[(t0 + t) * LC + c]);
+                        for (int t = 0; t < 8; ++t) s = cfma(s, l[t], s_y[(t0 + t) * LC + c]);
+                        acc[c] = cadd(acc[c], s);
+                    }
                 }
             } else {
                 for (int t = 0; t < jb; ++t) {
                     const C l = a[(size_t)t * n];
 #pragma unroll
-                    for (int c = 0; c < LC; ++c) acc[c] = cfms(acc[c], l, s_y[t * LC + c]);
+                    for (int c = 0; c < LC; ++c) acc[c] = cfma(acc[c], l, s_y[t * LC + c]);
                 }
             }
 #pragma unroll
             for (int c = 0; c < LC; ++c)
-                if (c < ncol) B[cb[c] + r] = acc[c];
+                if (c < ncol) B[cb[c] + r] = csub(B[cb[c] + r], acc[c]);
         }
         __syncthreads();
     };
