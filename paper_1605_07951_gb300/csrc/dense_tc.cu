@@ -33,7 +33,7 @@
 // stores to leave), all loads, half of A22's included, go out first, and the packing
 // behind them stores 16 bytes (4 of K') a lane with the eight lanes of a store phase on
 // consecutive rows (one element at a time, eight lanes met in a bank).  All updates of
-// 32 points of order 2048: 19.0 -> 10.0 ms; their 46 GB take 6.5 ms at copy rate.
+// 32 points of order 2048: 19.0 -> 10.0 ms; their 46 GB take 6.8 ms at copy rate.
 // The one mbarrier wait is bounded; a wait that runs out is counted in the
 // caller's status word and the tile is left unchanged.
 #include <algorithm>

@@ -364,7 +364,7 @@ RSRR_DEV void block_argmax(const double *__restrict__ d, int n, double &bv, int 
 // Column j costs n j complex FMAs on the FP64 unit: a block takes 32 rows, its
 // eight warps an eighth of the earlier columns each (a row per thread kept n /
 // 256 SMs busy), partial sums added in warp order.  The four factorisations of an
-// SS-RR solve of order 40000 with 2048 moment columns: 12.5 -> 4.1 ms, 3.5 ms with
+// RSRR solve of order 40000 with 2048 sample columns: 12.5 -> 4.1 ms, 3.5 ms with
 // the barrier of one atomic.
 __global__ void __launch_bounds__(256)
 pchol_persistent_kernel(const double2 *__restrict__ G, int n, double2 *__restrict__ Lm,
