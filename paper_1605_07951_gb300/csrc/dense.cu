@@ -664,10 +664,15 @@ dense_gemm_update_kernel(C *__restrict__ A_all, int n, int k0) {
 // -> 35.6 ms.  FP32: bound by reading the factor from L2 once per chunk, so the
 // chunks are as wide as leaves one for every SM: n = 2048, 64 right-hand sides,
 // 32 points 16.8 -> 5.4 ms for three solves, of which the last returns at once.
-// Since then a block's products are summed from zero (update; a solve 2.7 -> 3.1 ms):
-// subtracted one by one from the row they left 2.4 to 3.5 times the backward error
-// (random matrices of order 1200 and 2048, both precisions).
-template <typename C, int NB, int LC, int TH, bool IDENT>
+//
+// GROUP products at a time are summed from zero, then a block's sums, and the row
+// rounds once a block: subtracted one by one from the row they left 1.5 to 2.4 times
+// the backward error (random matrices of order 500 to 2048, both precisions; sphere
+// kernels 1.2 to 4 times).  By blocks (GROUP = NB) orders up to 500 are left with 1.0
+// to 1.1 times the error of sixteen partial sums, by eights with as much or less;
+// from about 1000 on both are below it, so by blocks there: n = 4096, 64 right-hand
+// sides, 32 points 9.4 ms a solve against 13.3 by eights and 9.3 one by one.
+template <typename C, int NB, int LC, int TH, bool IDENT, int GROUP>
 __global__ void __launch_bounds__(TH, 512 / TH)
 dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_all,
                    const C *__restrict__ dinv_all, C *__restrict__ B_all, int n, int L,
@@ -687,6 +692,7 @@ dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_
     __shared__ __align__(16) C s_y[NB * LC];
     __shared__ int s_col[LC], s_dst[2 * NB], s_src[2 * NB], s_moves;
     static_assert(!IDENT || NB % LC == 0, "a chunk's ones lie in one block");
+    static_assert(GROUP == 8 || GROUP == NB, "the loads go by eights");
     extern __shared__ int s_perm[];  // IDENT: position -> row, then the pivots
     if (IDENT) {
         // the interchanges composed: row s_perm[p] ends at position p
@@ -737,14 +743,16 @@ dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_
         }
         __syncthreads();
     };
-    // rows r_lo .. r_hi-1 -= A(:, k0 .. k0+jb-1) y: eight products at a time summed from
-    // zero, then a block's sums, so that they round by their own size and the row rounds
-    // once a block
+    // rows r_lo .. r_hi-1 -= A(:, k0 .. k0+jb-1) y
     auto update = [&](int k0, int jb, int r_lo, int r_hi) {
+        constexpr bool EARLY = GROUP == NB;  // the row's values first: room in the registers
         for (int r = r_lo + tid; r < r_hi; r += TH) {
-            C acc[LC];
+            C acc[LC], b[EARLY ? LC : 1];
 #pragma unroll
-            for (int c = 0; c < LC; ++c) acc[c] = czero<C>();
+            for (int c = 0; c < LC; ++c) {
+                acc[c] = czero<C>();
+                if constexpr (EARLY) b[c] = c < ncol ? B[cb[c] + r] : czero<C>();
+            }
             const C *a = A + (size_t)k0 * n + r;
             if (jb == NB) {
 #pragma unroll 1
@@ -752,12 +760,19 @@ dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_
                     C l[8];
 #pragma unroll
                     for (int t = 0; t < 8; ++t) l[t] = a[(size_t)(t0 + t) * n];
+                    if constexpr (GROUP == NB) {
 #pragma unroll
-                    for (int c = 0; c < LC; ++c) {
-                        C s = czero<C>();
+                        for (int t = 0; t < 8; ++t)
 #pragma unroll
-                        for (int t = 0; t < 8; ++t) s = cfma(s, l[t], s_y[(t0 + t) * LC + c]);
-                        acc[c] = cadd(acc[c], s);
+                            for (int c = 0; c < LC; ++c) acc[c] = cfma(acc[c], l[t], s_y[(t0 + t) * LC + c]);
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < LC; ++c) {
+                            C s = czero<C>();
+#pragma unroll
+                            for (int t = 0; t < 8; ++t) s = cfma(s, l[t], s_y[(t0 + t) * LC + c]);
+                            acc[c] = cadd(acc[c], s);
+                        }
                     }
                 }
             } else {
@@ -769,7 +784,7 @@ dense_solve_kernel(const C *__restrict__ A_all, const int32_t *__restrict__ piv_
             }
 #pragma unroll
             for (int c = 0; c < LC; ++c)
-                if (c < ncol) B[cb[c] + r] = csub(B[cb[c] + r], acc[c]);
+                if (c < ncol) B[cb[c] + r] = csub(EARLY ? b[EARLY ? c : 0] : B[cb[c] + r], acc[c]);
         }
         __syncthreads();
     };
@@ -1114,12 +1129,15 @@ static int ds_columns(int N, int L, int widest) {
         if ((int64_t)N * ((L + lc - 1) / lc) >= sms * 4 / 5) return lc;
     return 4;
 }
+constexpr int DS_GROUPED = 1024;  // largest order whose products are summed by eights
 template <typename C, int NB, int LC, int TH>
 static cudaError_t ds_launch(const C *A, const int32_t *piv, const C *dinv, C *B, int n, int N, int L,
                              const int32_t *skip, cudaStream_t s) {
+    auto *kernel = n <= DS_GROUPED ? dense_solve_kernel<C, NB, LC, TH, false, 8>
+                                   : dense_solve_kernel<C, NB, LC, TH, false, NB>;
     for (int p0 = 0; p0 < N; p0 += 65535) {  // grid.y limit
         const size_t nblk = ((size_t)n + NB - 1) / NB;
-        dense_solve_kernel<C, NB, LC, TH, false><<<dim3((L + LC - 1) / LC, std::min(N - p0, 65535)), TH, 0, s>>>(
+        kernel<<<dim3((L + LC - 1) / LC, std::min(N - p0, 65535)), TH, 0, s>>>(
             A + (size_t)p0 * n * n, piv + (size_t)p0 * n, dinv + p0 * nblk * 2 * NB * NB, B + (size_t)p0 * n * L, n, L,
             skip ? skip + p0 : nullptr);
     }
@@ -1162,7 +1180,7 @@ cudaError_t launch_dense_inverse_c128(const double2 *A, const int32_t *piv, cons
             if (e != cudaSuccess) return e;
             continue;
         }
-        dense_solve_kernel<double2, NB_C128, LC, TH, true>
+        dense_solve_kernel<double2, NB_C128, LC, TH, true, 8>
             <<<dim3((n + LC - 1) / LC, np), TH, sizeof(int) * (size_t)(2 * n), s>>>(
                 A + p0 * nn, piv + (size_t)p0 * n, dinv + p0 * nblk * 2 * NB_C128 * NB_C128, X + p0 * nn, n, n,
                 nullptr);
